@@ -79,49 +79,94 @@ __global__ void scatter_rows_kernel(int32_t *dst, const int64_t *idx, const int3
         dst[idx[i / DEG] * DEG + (i % DEG)] = rows[i];
 }
 
+// ||a - b||^2 of decoded vectors in the host build's float arithmetic, one pair per group of
+// eight lanes (four pairs per warp).  The host sums eight partials (s_u over the coordinates
+// t = u mod 8 of the full groups of eight, the remaining coordinates onto s_0) and adds them
+// as ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)), every operation rounded on its own:
+// lane u of a group keeps s_u and the tree is three butterfly adds, so the result is the host's
+// bit for bit, and a group reads 32 consecutive bytes of each vector at a time.
+// OctVec: this lane's share of one vector (coordinates u, u + 8, ...; NG full groups of eight,
+// NG = 0: read from memory at each use, for other d).
+template <int NG>
+struct OctVec {
+    float x[NG > 0 ? NG : 1];
+    const float *p;
+    __device__ __forceinline__ void load(const float *row, int lane)
+    {
+        p = row;
+        if constexpr (NG > 0) {
+#pragma unroll
+            for (int g = 0; g < NG; g++) x[g] = __ldg(row + 8 * g + (lane & 7));
+        }
+    }
+};
+
+template <int NG>
+__device__ __forceinline__ float oct_l2(const OctVec<NG> &a, const float *b, int d, int lane)
+{
+    const int u = lane & 7;
+    float s = 0.f;
+    if constexpr (NG > 0) {
+        float y[NG];
+#pragma unroll
+        for (int g = 0; g < NG; g++) y[g] = __ldg(b + 8 * g + u);
+#pragma unroll
+        for (int g = 0; g < NG; g++) {
+            const float x = __fsub_rn(a.x[g], y[g]);
+            s = __fadd_rn(s, __fmul_rn(x, x));
+        }
+    } else {
+        int t = 0;
+        for (; t + 8 <= d; t += 8) {
+            const float x = __fsub_rn(__ldg(a.p + t + u), __ldg(b + t + u));
+            s = __fadd_rn(s, __fmul_rn(x, x));
+        }
+        if (u == 0)
+            for (; t < d; t++) {
+                const float x = __fsub_rn(__ldg(a.p + t), __ldg(b + t));
+                s = __fadd_rn(s, __fmul_rn(x, x));
+            }
+    }
+    s = __fadd_rn(s, __shfl_xor_sync(FULL, s, 1));
+    s = __fadd_rn(s, __shfl_xor_sync(FULL, s, 2));
+    return __fadd_rn(s, __shfl_xor_sync(FULL, s, 4));
+}
+
+// Whether some of the first `kept` entries of kid (lane u holds the u-th) is closer to the
+// candidate v than `dist` (warp-uniform): four entries at a time, stopping at the first that is.
+template <int NG>
+__device__ __forceinline__ bool any_closer(const OctVec<NG> &v, float dist, int32_t kid, int kept, const float *xh,
+                                           int d, int lane)
+{
+    for (int k0 = 0; k0 < kept; k0 += 4) {
+        const int k = k0 + (lane >> 3);
+        const int32_t id = __shfl_sync(FULL, kid, min(k, kept - 1));
+        const float dk = oct_l2<NG>(v, xh + (int64_t)id * d, d, lane);
+        if (__ballot_sync(FULL, k < kept && dk < dist)) return true;
+    }
+    return false;
+}
+
 // Neighbour selection of the GPU-assisted build: HNSW's shrinking heuristic on each member's
 // candidate list (sorted by distance to the member): a candidate is kept unless it is closer to
-// an already kept neighbour than to the member, up to DEG kept.  One warp per member; lane u
-// tests the candidate against the u-th kept neighbour.  The decoded-to-decoded distance
-// reproduces the host build's float arithmetic (eight partial sums over coordinate groups,
-// then a fixed tree; no multiply-add contraction), so the choices are the host's.
+// an already kept neighbour than to the member, up to DEG kept.  One warp per member.  The
+// decoded-to-decoded distances are the host build's (above), so the choices are the host's.
+// What bounds it is the latency of 40 dependent candidate tests, so the next candidate's vector
+// is loaded while the current one is tested, and each test reads the decoded vectors (held on
+// the device for the linking) with eight lanes per pair.  Decoding both vectors coordinate by
+// coordinate from the codebooks, one pair per lane, took 555 us per launch (mean over the 159
+// launches of a 60,000-vector add); 27.6 us now.
 struct SelectArgs {
     const int32_t *cand_ids;          // [m][efc], -1 padded
     const float *cand_d;              // [m][efc]
     int32_t *sel;                     // [m][DEG + 1]: kept ids, then their count
     int64_t m;
-    int efc, d, M1, M2P;
-    const float *C1, *C2;
-    const uint8_t *codes1, *codes2b;
-    uint8_t sub1[256], sub2[256];
+    int efc, d;
+    const float *xh;                  // [n][d] decoded vectors
 };
 
-__device__ __forceinline__ float decoded_at(const SelectArgs &a, int32_t v, int t)
-{
-    return __fadd_rn(__ldg(a.C1 + (int)__ldg(a.codes1 + (int64_t)v * a.M1 + a.sub1[t]) * a.d + t),
-                     __ldg(a.C2 + (int)__ldg(a.codes2b + (int64_t)v * a.M2P + a.sub2[t]) * a.d + t));
-}
-
-__device__ float decoded_l2(const SelectArgs &a, int32_t p, int32_t q)
-{
-    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int t = 0;
-    for (; t + 8 <= a.d; t += 8) {
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-            const float x = __fsub_rn(decoded_at(a, p, t + u), decoded_at(a, q, t + u));
-            s[u] = __fadd_rn(s[u], __fmul_rn(x, x));
-        }
-    }
-    for (; t < a.d; t++) {
-        const float x = __fsub_rn(decoded_at(a, p, t), decoded_at(a, q, t));
-        s[0] = __fadd_rn(s[0], __fmul_rn(x, x));
-    }
-    return __fadd_rn(__fadd_rn(__fadd_rn(s[0], s[1]), __fadd_rn(s[2], s[3])),
-                     __fadd_rn(__fadd_rn(s[4], s[5]), __fadd_rn(s[6], s[7])));
-}
-
-__global__ void __launch_bounds__(256) select_kernel(const SelectArgs a)
+template <int NG>
+__global__ void __launch_bounds__(128) select_kernel(const SelectArgs a)
 {
     const int lane = threadIdx.x & 31;
     const int64_t mi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -130,15 +175,22 @@ __global__ void __launch_bounds__(256) select_kernel(const SelectArgs a)
     const float *cd = a.cand_d + mi * a.efc;
     int kept = 0;
     int32_t kid = -1;                                    // lane u: the u-th kept neighbour
-    for (int s = 0; s < a.efc && kept < DEG; s++) {
-        const int32_t c = __ldg(ci + s);
-        if (c < 0) break;
-        const float dc = __ldg(cd + s);
-        const bool closer = lane < kept && decoded_l2(a, c, kid) < dc;
-        if (__ballot_sync(FULL, closer) == 0) {
+    int32_t c = __ldg(ci);
+    float dc = __ldg(cd);
+    OctVec<NG> v;
+    if (c >= 0) v.load(a.xh + (int64_t)c * a.d, lane);
+    for (int s = 0; s < a.efc && kept < DEG && c >= 0; s++) {
+        const int32_t c1 = s + 1 < a.efc ? __ldg(ci + s + 1) : -1;
+        const float dc1 = s + 1 < a.efc ? __ldg(cd + s + 1) : 0.f;
+        OctVec<NG> v1;
+        if (c1 >= 0) v1.load(a.xh + (int64_t)c1 * a.d, lane);
+        if (!any_closer<NG>(v, dc, kid, kept, a.xh, a.d, lane)) {
             if (lane == kept) kid = c;
             kept++;
         }
+        c = c1;
+        dc = dc1;
+        v = v1;
     }
     int32_t *out = a.sel + mi * (DEG + 1);
     out[lane] = lane < kept ? kid : -1;
@@ -199,14 +251,9 @@ lc_status build_gpu_select_start(lc_index *ix, const float *xr, int64_t m, int e
     }
     SelectArgs sa{};
     sa.cand_ids = dv->b_ids; sa.cand_d = dv->b_d; sa.sel = dv->b_sel; sa.m = m; sa.efc = efc;
-    sa.d = dv->d; sa.M1 = dv->M1; sa.M2P = dv->M2P; sa.C1 = dv->C1; sa.C2 = dv->C2;
-    sa.codes1 = dv->codes1; sa.codes2b = dv->codes2b;
-    std::vector<int> o, l;
-    splits(dv->d, dv->M1, o, l);
-    for (int j = 0; j < dv->M1; j++) for (int t = o[j]; t < o[j] + l[j]; t++) sa.sub1[t] = (uint8_t)j;
-    splits(dv->d, dv->M2, o, l);
-    for (int j = 0; j < dv->M2; j++) for (int t = o[j]; t < o[j] + l[j]; t++) sa.sub2[t] = (uint8_t)j;
-    select_kernel<<<(unsigned)((m * 32 + 255) / 256), 256>>>(sa);
+    sa.d = dv->d; sa.xh = lk->xh;
+    const auto kern = dv->d == 96 ? select_kernel<12> : dv->d == 128 ? select_kernel<16> : select_kernel<0>;
+    kern<<<(unsigned)((m * 32 + 127) / 128), 128>>>(sa);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(lk->h_buf, dv->b_sel, sizeof(int32_t) * m * (DEG + 1), cudaMemcpyDeviceToHost, 0) != cudaSuccess ||
         cudaMemcpyAsync(lk->h_status, dv->status, sizeof(int32_t), cudaMemcpyDeviceToHost, 0) != cudaSuccess) {
@@ -630,21 +677,25 @@ __global__ void __launch_bounds__(256) own_rows_kernel(const Link0Args a)
 }
 
 // One warp per target: lane s holds entry s of the row (packed: valid entries first, in
-// (distance, id) order).
-__global__ void __launch_bounds__(256) links_kernel(const Link0Args a)
+// (distance, id) order).  Bound by the latency of the dependent distance tests; the distances
+// take eight lanes per pair (oct_l2), as in select_kernel: 80.3 us per launch with one pair per
+// lane, 41.8 us now (mean over the 160 launches of a 60,000-vector add).
+template <int NG>
+__global__ void __launch_bounds__(128) links_kernel(const Link0Args a)
 {
     const int lane = threadIdx.x & 31;
     const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (g >= a.G) return;                                // whole warps leave together
     const int64_t t = __ldg(a.targets + g);
-    const float *xt = a.xh + t * a.d;
+    OctVec<NG> xt;
+    xt.load(a.xh + t * a.d, lane);
     int32_t id = a.adj0[t * DEG + lane];
     float dd = a.adj0d[t * DEG + lane];
     const int i1 = __ldg(a.starts + g + 1);
     for (int i = __ldg(a.starts + g); i < i1; i++) {
         const int32_t x = __ldg(a.src + i);
         if (__ballot_sync(FULL, id == x)) continue;      // already linked
-        const float kd = l2_decoded(xt, a.xh + (int64_t)x * a.d, a.d);
+        const float kd = oct_l2<NG>(xt, a.xh + (int64_t)x * a.d, a.d, lane);
         const bool valid = id >= 0;
         const int n = __popc(__ballot_sync(FULL, valid));
         const int pos = __popc(__ballot_sync(FULL, valid && key_less(dd, id, kd, x)));
@@ -667,8 +718,9 @@ __global__ void __launch_bounds__(256) links_kernel(const Link0Args a)
         for (int c = 0; c <= DEG && kept < DEG; c++) {
             const int32_t sid = c < DEG ? __shfl_sync(FULL, cid, c) : last_id;
             const float sd = c < DEG ? __shfl_sync(FULL, cd, c) : last_d;
-            const bool closer = lane < kept && l2_decoded(a.xh + (int64_t)sid * a.d, a.xh + (int64_t)kid * a.d, a.d) < sd;
-            if (__ballot_sync(FULL, closer) == 0) {
+            OctVec<NG> v;
+            v.load(a.xh + (int64_t)sid * a.d, lane);
+            if (!any_closer<NG>(v, sd, kid, kept, a.xh, a.d, lane)) {
                 if (lane == kept) { kid = sid; kdd = sd; }
                 kept++;
             }
@@ -762,7 +814,8 @@ lc_status build_gpu_link0(lc_index *ix, int64_t first, int64_t b, const int32_t 
     // members' rows first, then the back-links (disjoint rows: a member is never a target of
     // its own batch, whose searches saw the graph as it stood at the batch start)
     own_rows_kernel<<<(unsigned)((b * 32 + 255) / 256), 256>>>(a);
-    if (G > 0) links_kernel<<<(unsigned)((G * 32 + 255) / 256), 256>>>(a);
+    const auto links = a.d == 96 ? links_kernel<12> : a.d == 128 ? links_kernel<16> : links_kernel<0>;
+    if (G > 0) links<<<(unsigned)((G * 32 + 127) / 128), 128>>>(a);
     const int grid = (int)std::min<int64_t>((R * DEG + 255) / 256, (int64_t)dv->num_sms * 8);
     gather_rows_kernel<<<std::max(grid, 1), 256>>>(dv->adj0, lk->ridx, R, lk->rid);
     // the ids come back (the host searches of later batches read them); the row distances
