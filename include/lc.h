@@ -115,7 +115,7 @@ typedef struct {
     int max_dist;    /* search-time cap T (Section 3.1): 0 = none; > 0: the level-0 search stops
                         before an expansion once T distances have been computed there */
     int warps;       /* walk queries in flight per thread block: 0 = as many as fit in shared
-                        memory (at most 16); 1..16 = at most that many.  Results do not depend
+                        memory (at most 24); 1..16 = at most that many.  Results do not depend
                         on it (a launch-shape knob for the autotuner) */
     int walk_full;   /* 0: the walk scores the level-1 code by ADC (the default reading of
                         Section 4.1); 1: it scores the full two-level decode q = c1 + c2 (each

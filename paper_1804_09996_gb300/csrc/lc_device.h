@@ -87,6 +87,25 @@ inline bool grow(T *&p, size_t &cap, size_t need)
     return true;
 }
 
+// The visited set of one query.  Its limits are those of a shared table of 2^hash_log ids,
+// taken to three quarters, and then a global one of 2^spill_log, taken to half: a row of 32
+// neighbours that would pass the second limit fails the query.  The limits are counted as such
+// whatever the storage, which is 16-byte buckets, each read by one 16-byte load:
+//   tag = 1: eight 16-bit tags per bucket.  An id below 2^nb is multiplied by an odd constant
+//     modulo 2^nb (a bijection): the top bb bits of the product choose the bucket, the other
+//     tb = nb - bb <= 16 bits (plus one below 16 bits; 0 = empty) are the tag, so the tag
+//     identifies the id exactly.  An id whose bucket is full (or whose tag is 0) goes to a small table
+//     of ids in shared memory (2^stash_log entries) and, once that is three quarters full, to the
+//     global table.  Half the bytes of the ids per entry: a walk's table takes 4.5 KB and not 8,
+//     so that up to 24 walks fit on an SM and not 16.
+//   tag = 0: four 32-bit ids (plus one) per bucket, a full bucket continuing in the next, the
+//     global table behind; for indexes too large for the tags and for the table sizes that a
+//     caller asks for.
+struct VisitTab {
+    int tag, bb, tb, stash_log;
+    uint32_t mul, bytes;           // multiplier, bytes of the buckets
+};
+
 // Launch configuration of one search and the scratch it needs.
 struct SearchPlan {
     int k = 0, efp = 0, R = 0, beam = 1, tcap = 0, hash_log = 0, spill_log = 0, variant = 0;
@@ -105,6 +124,8 @@ struct SearchPlan {
     size_t tab_elems = 0;                // FP16 table entries of the batch
     int dwpc = 0, dgrid = 0;             // ordered search: the descent launch's warps per CTA, CTAs
     size_t dsmem = 0;
+    VisitTab vt{};                       // visited set in shared memory
+    int64_t spill_tables = 0;            // global visited tables
     size_t yq_elems = 0, sl_elems = 0, spill_elems = 0, ord_elems = 0;
 };
 
@@ -112,7 +133,7 @@ struct SearchPlan {
 struct SearchScratch {
     float *yq = nullptr;                 // [nq][d] rotated queries
     int32_t *shortlist = nullptr;        // [nq][R] (refinement only)
-    int32_t *spill = nullptr;            // [grid * wpc][2^spill_log]
+    int32_t *spill = nullptr;            // [spill_tables][2^spill_log]
     uint16_t *tab = nullptr;             // table form: [nq][256][32] FP16
     int32_t *ord = nullptr;              // ordered search: entry node, upper evaluations, queue
                                          // order (int32) and entry distance (float), [nq] each

@@ -213,11 +213,14 @@ __global__ void __launch_bounds__(TAB_WARPS * 32) table_kernel(const float *yq, 
                                                                __half *T)
 {
     constexpr int M1 = TAB_M1, D = 96;
-    // the FP16 codebook in the walk's split layout: half2 [256][32] (coordinates 0, 1 of every
-    // sub-space), then half [256][32] (coordinate 2)
+    // the FP16 codebook, which the walk keeps as four halves per (centroid, sub-space), as half2
+    // [256][32] (coordinates 0, 1 of every sub-space), then half [256][32] (coordinate 2)
     __shared__ __align__(16) __half cb[256 * M1 * 3];
-    for (int i = threadIdx.x; i < 256 * M1 * 3 / 8; i += blockDim.x)
-        reinterpret_cast<uint4 *>(cb)[i] = __ldg(reinterpret_cast<const uint4 *>(C1h) + i);
+    for (int i = threadIdx.x; i < 256 * M1; i += blockDim.x) {
+        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(C1h) + i);
+        reinterpret_cast<uint32_t *>(cb)[i] = w.x;
+        cb[256 * M1 * 2 + i] = __ushort_as_half((unsigned short)(w.y & 0xffff));
+    }
     __syncthreads();
     const __half2 *cb2 = reinterpret_cast<const __half2 *>(cb);
     const __half *cb1 = cb + 256 * M1 * 2;
@@ -556,16 +559,19 @@ lc_status upload(lc_index *ix)
                 for (int u = 0; u < sl[j]; u++) {
                     const float v = ix->C1[(size_t)c * d + so[j] + u];
                     if (L == 0) put((size_t)c * d + so[j] + u, v);
-                    else if (L == 1) put(((size_t)c * M1 + j) * P + u, v);
-                    else put(u < 2 ? ((size_t)c * M1 + j) * 2 + u : (size_t)256 * M1 * 2 + (size_t)c * M1 + j, v);
+                    else put(((size_t)c * M1 + j) * P + u, v);
                 }
     };
     std::vector<float> c1w(walk_c1_bytes(d, M1, D1, 4) / 4, 0.f);
     put_layout(4, [&](size_t i, float v) { c1w[i] = v; });
     std::vector<__half> c1h(walk_c1_bytes(d, M1, D1, 2) / 2, __float2half_rn(0.f));
     put_layout(2, [&](size_t i, float v) { c1h[i] = __float2half_rn(v); });
-    std::vector<__half> c2h(ix->C2.size());
-    for (size_t i = 0; i < c2h.size(); i++) c2h[i] = __float2half_rn(ix->C2[i]);   // round to nearest even
+    // the level-2 one rounded likewise, in the full walk's layout
+    std::vector<__half> c2h(walk_c2_bytes(d, M1, D1) / 2, __float2half_rn(0.f));
+    for (int c = 0; c < 256; c++)
+        for (int t = 0; t < d; t++)
+            c2h[walk_c2_lanes(D1, 2) ? ((size_t)c * M1 + t / D1) * walk_pad(D1) + t % D1 : (size_t)c * d + t] =
+                __float2half_rn(ix->C2[(size_t)c * d + t]);
     __half *c2h_dev = static_cast<__half *>(dv->C2h);
     __half *c1h_dev = static_cast<__half *>(dv->C1h);
     bool ok = dupload(dv->Rt, Rt) && dupload(dv->C1, ix->C1) && dupload(dv->C2, ix->C2) &&
@@ -654,19 +660,33 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
                   "M1 = 64 at d = 128); use FP32");
         return LC_ERR_ARG;
     }
-    P.per_warp = walk_smem(dv->M1, dv->d, efcap, P.hash_log, P.beam, false, P.full ? dv->M2P : 0).total;
-    WalkArgs wa{};
-    wa.nq = nq;
-    wa.d = dv->d;
+    const int m2p = P.full ? dv->M2P : 0;
     P.tab = sp->lut_prec == LC_LUT_TABLE;
     if (P.tab && (P.variant != 2 || P.full)) {
         set_error("the table form is built for 32 level-1 sub-spaces of 3 coordinates (d = 96) and the level-1 walk");
         return LC_ERR_ARG;
     }
     P.half = sp->lut_prec == LC_LUT_FP16 || P.tab;
+    // shared memory of a CTA: the codebook (or, per walk, the query's table) and the walks.  A search
+    // too wide for it is refused by the size of its limits (walk_smem_nominal)
+    const size_t tab_b = P.tab ? (size_t)256 * TAB_M1 * 2 : 0;
+    const size_t cb_b = P.tab ? 0 : walk_cb_bytes(dv->d, dv->M1, walk_variant_d1(P.variant), P.half ? 2 : 4, P.full);
+    const size_t nominal = (P.tab ? tab_b : walk_nominal_cb_bytes(dv->d, dv->M1, P.half, P.full)) +
+                           walk_smem_nominal(dv->M1, dv->d, efcap, P.hash_log, P.beam, false, m2p);
+    bool fits = nominal <= MAX_SMEM_PER_BLOCK;
+    P.vt = visit_tab(dv->n, P.hash_log, sp->visited_log == 0 && sp->spill_log == 0);
+    P.per_warp = tab_b + walk_smem(dv->M1, dv->d, efcap, P.vt, P.beam, false, m2p).total;
+    if (fits && P.vt.tag && cb_b + P.per_warp > MAX_SMEM_PER_BLOCK) {
+        P.vt = visit_tab(dv->n, P.hash_log, false);
+        P.per_warp = tab_b + walk_smem(dv->M1, dv->d, efcap, P.vt, P.beam, false, m2p).total;
+    }
+    WalkArgs wa{};
+    wa.nq = nq;
+    wa.d = dv->d;
     cudaError_t ce;
-    if (P.tab) {
-        P.per_warp += (size_t)256 * TAB_M1 * 2;                 // the query's table
+    if (!fits) {
+        ce = cudaErrorInvalidConfiguration;
+    } else if (P.tab) {
         P.tab_elems = (size_t)nq * 256 * TAB_M1;
         ce = walk_config_tab(wa, P.per_warp, dv->num_sms, sp->warps, &P.wpc, &P.grid, &P.smem);
     } else {
@@ -684,7 +704,9 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
                   cudaGetErrorString(ce));
         return LC_ERR_CUDA;
     }
-    P.spill_elems = ((size_t)P.grid * P.wpc) << P.spill_log;
+    // one global visited table per query, or per walk in flight where there are more queries
+    P.spill_tables = std::min<int64_t>(nq, (int64_t)P.grid * P.wpc);
+    P.spill_elems = (size_t)P.spill_tables << P.spill_log;
     P.yq_elems = (size_t)nq * dv->d;
     // ordered search: worth its two extra launches once every warp takes a few queries
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
@@ -758,7 +780,9 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     wa.tcap = P.tcap;
     wa.hash_log = P.hash_log;
     wa.spill_log = P.spill_log;
+    wa.vt = P.vt;
     wa.spill = sc.spill;
+    wa.spill_tables = P.spill_tables;
     wa.status = sc.status;
     wa.counter = sc.counter;
     wa.stats_out = dstats;
@@ -811,7 +835,6 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
         int32_t *seed = sc.ord, *seed_up = sc.ord + nq, *order = sc.ord + 2 * nq;
         float *seed_d = reinterpret_cast<float *>(sc.ord + 3 * nq);
         WalkArgs w1 = wa;
-        w1.mode = 1;
         w1.seed = seed;
         w1.seed_up = seed_up;
         w1.seed_d = seed_d;
@@ -1105,19 +1128,29 @@ lc_status search_walk_noalloc(lc_index *ix, const float *q, int64_t nq, int k, i
     std::vector<int> off, len;
     splits(dv->d, dv->M1, off, len);
     for (int j = 0; j < dv->M1; j++) { wa.s1.off[j] = (uint16_t)off[j]; wa.s1.len[j] = (uint8_t)len[j]; }
-    const size_t per_warp = walk_smem(dv->M1, dv->d, wa.efcap, wa.hash_log, wa.beam, true).total;
+    wa.vt = visit_tab(dv->n, wa.hash_log, true);
+    const size_t cb_b = walk_cb_bytes(dv->d, dv->M1, walk_variant_d1(walk_variant(dv->M1, dv->d)), 4, false);
+    if (cb_b + walk_smem(dv->M1, dv->d, wa.efcap, wa.vt, wa.beam, true).total > MAX_SMEM_PER_BLOCK)
+        wa.vt = visit_tab(dv->n, wa.hash_log, false);
+    const size_t per_warp = walk_smem(dv->M1, dv->d, wa.efcap, wa.vt, wa.beam, true).total;
+    if (walk_nominal_cb_bytes(dv->d, dv->M1, false, false) +
+            walk_smem_nominal(dv->M1, dv->d, wa.efcap, wa.hash_log, wa.beam, true) > MAX_SMEM_PER_BLOCK) {
+        set_error("walk kernel configuration failed: %s", cudaGetErrorString(cudaErrorInvalidConfiguration));
+        return LC_ERR_CAPACITY;
+    }
     const int variant = (dv->M1 == 16 && dv->d == 96) ? 1 : (dv->M1 == 32 && dv->d == 96) ? 2
                       : (dv->M1 == 64 && dv->d == 128) ? 3 : 0;
     int grid = 0, wpc = 1;
     size_t smem = 0;
     cudaError_t ce;
-    ce = walk_config(false, variant, dv->M1, false, wa, per_warp, dv->num_sms, 0, &wpc, &grid, &smem);
+    // every warp in flight owns one spill table of the array
+    const size_t slots = NOALLOC_SPILL_BYTES / ((size_t)4 << wa.spill_log);
+    const int want = (int)std::max<size_t>(1, slots / std::max(1, dv->num_sms));     // all SMs before more walks on each
+    ce = walk_config(false, variant, dv->M1, false, wa, per_warp, dv->num_sms, want, &wpc, &grid, &smem);
     if (ce != cudaSuccess) {
         set_error("walk kernel configuration failed: %s", cudaGetErrorString(ce));
         return ce == cudaErrorInvalidConfiguration ? LC_ERR_CAPACITY : LC_ERR_CUDA;
     }
-    // every warp in flight owns one spill table of the array
-    const size_t slots = NOALLOC_SPILL_BYTES / ((size_t)4 << wa.spill_log);
     grid = (int)std::min<int64_t>(grid, (int64_t)(slots / wpc));
     // the array keeps the previous call's contents: the counter and status start at zero
     // (spill tables are cleared by the kernel before a query uses one)
@@ -1125,6 +1158,7 @@ lc_status search_walk_noalloc(lc_index *ix, const float *q, int64_t nq, int k, i
         set_error("reset of the no-allocation scratch failed: %s", cudaGetErrorString(cudaGetLastError()));
         return LC_ERR_CUDA;
     }
+    wa.spill_tables = (int64_t)grid * wpc;
     ce = walk_run(false, variant, dv->M1, false, wa, smem, wpc, grid, st);
     if (ce != cudaSuccess) {
         set_error("walk kernel launch failed: %s", cudaGetErrorString(ce));

@@ -170,10 +170,16 @@ lc_status plan_batch(lc_server *s, Batch &b)
         b.nq += r->nq;
     }
     b.sp.ef = efb;                              // the bound of the per-query efSearch
-    lc_status rs = lc::plan_search(s->dv, b.nq, &b.sp, &b.plan, true);
-    if (rs != LC_OK) return rs;
-    layout(b, s->dv->d);
-    return LC_OK;
+    // a lone request whose walks in flight would need more visited tables than the budget holds
+    // runs with fewer walks at a time (results do not depend on it)
+    for (int warps = b.reqs[0]->sp.warps;;) {
+        b.sp.warps = warps;
+        lc_status rs = lc::plan_search(s->dv, b.nq, &b.sp, &b.plan, true);
+        if (rs != LC_OK) return rs;
+        layout(b, s->dv->d);
+        if (b.need <= s->budget || b.reqs.size() > 1 || b.plan.wpc == 1) return LC_OK;
+        warps = b.plan.wpc > 16 ? 16 : b.plan.wpc / 2;
+    }
 }
 
 void deliver(lc_server *s, lc_server::Slot &sl, lc_status status)

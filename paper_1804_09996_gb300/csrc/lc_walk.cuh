@@ -17,8 +17,8 @@
 //     once (one per lane) and merges them into W keeping the ef' best.  With one expansion
 //     per step this expands exactly the nodes, in exactly the order, of the two-set
 //     formulation (candidate heap C + result heap W);
-//   - exact visited set: open-addressing hash in shared memory, spilling to a per-warp table
-//     in global memory when it fills;
+//   - exact visited set: 16-byte buckets in shared memory (eight 16-bit tags or four ids each),
+//     with a per-warp table in global memory behind it;
 //   - writes the shortlist (the R best of W, Section 4.1 two-stage search) or, without
 //     refinement, the top-k directly;
 //   - ordered search: a first launch (mode 1) runs only the upper-level descent of every query
@@ -48,6 +48,39 @@ namespace lc {
 #define FULL 0xffffffffu
 
 // ------------------------------------------------------------------------------------------
+// Visited set (VisitTab in lc_device.h)
+constexpr uint32_t VISIT_MUL = 0x9E3779B1u;
+
+// The storage for an index of n ids, limits of 2^hash_log; want_tag: tags where they fit.
+inline VisitTab visit_tab(int64_t n, int hash_log, bool want_tag)
+{
+    int nb = 1;
+    while (nb < 31 && ((int64_t)1 << nb) < n) nb++;
+    VisitTab v{};
+    for (int h = hash_log; want_tag && h <= hash_log + 1; h++) {
+        const int bb = h - 3;                             // 8 tags per bucket
+        nb = nb <= bb ? bb + 1 : nb;
+        if (nb - bb > 16) continue;                       // one more bit of buckets: as large as with ids
+        v.tag = 1;
+        v.bb = bb;
+        v.tb = nb - bb;
+        v.mul = VISIT_MUL << (32 - nb);
+        v.bytes = 16u << bb;
+        v.stash_log = h - 4;
+        return v;
+    }
+    v.bb = hash_log - 2;                                  // 4 ids per bucket
+    v.mul = VISIT_MUL;
+    v.bytes = 16u << v.bb;
+    v.stash_log = -1;
+    return v;
+}
+__host__ __device__ inline size_t visit_bytes(const VisitTab &v)
+{
+    return v.bytes + (v.stash_log >= 0 ? (size_t)4 << v.stash_log : 0);
+}
+constexpr uint32_t OWNERS = 512;         // owner bytes of visit_rows (in the staging area, unused then)
+
 // Kernel arguments
 struct SplitTab {
     uint16_t off[64];
@@ -73,9 +106,11 @@ struct WalkArgs {
     int refine;
     int beam;         // expansions per step (1: the plain walk)
     int tcap;         // > 0: stop once that many level-0 distances were computed
-    int hash_log;     // shared-memory visited table: 2^hash_log entries
-    int spill_log;    // global spill table per warp: 2^spill_log entries
+    int hash_log;     // visited-set limits: 2^hash_log entries (see VisitTab) ...
+    int spill_log;    // ... and a global table of 2^spill_log entries per query in flight
+    VisitTab vt;      // the shared-memory part
     int32_t *spill;
+    int64_t spill_tables;  // tables behind spill: one per query (nq) or one per warp
     const float *yq_in;    // non-null: y' = R y computed by rotate_kernel (read, not recomputed)
     float *yq_out;
     int32_t *short_out;
@@ -91,10 +126,10 @@ struct WalkArgs {
     const uint8_t *codes2b;
     int M2P;
     uint8_t sub2[256];     // level-2 sub-space of each coordinate
-    // ordered search (see walk_kernel): 0 = the whole walk; 1 = the upper levels only, writing
-    // each query's level-0 entry node, its walk distance and the upper-level evaluations to
-    // seed / seed_d / seed_up; 2 = level 0 only, from those, queue position i taking query
-    // order[i] (order may be null: position i is query i)
+    // ordered search: descent_kernel writes each query's level-0 entry node, its walk distance
+    // and the upper-level evaluations to seed / seed_d / seed_up.  walk_kernel: 0 = the whole
+    // walk; 2 = level 0 only, from those, queue position i taking query order[i] (order may be
+    // null: position i is query i)
     int mode;
     const int32_t *order;
     const __half *tab;     // table form: the queries' ADC tables [nq][256][M1] (FP16)
@@ -102,14 +137,20 @@ struct WalkArgs {
     float *seed_d;
 };
 
-constexpr int MAX_WALK_WARPS = 16;       // warps (queries in flight) per CTA
+constexpr int MAX_WALK_WARPS = 20;       // warps (queries in flight) per CTA
+// threads per CTA an instantiation is compiled for: the full-decode walk and the uneven splits
+// keep more per-lane state, so they get registers for 16 warps
+__host__ __device__ constexpr int walk_threads(int D1, bool fq)
+{
+    return (fq || D1 == 0 ? 16 : MAX_WALK_WARPS) * 32;
+}
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Shared memory of the walk kernel: the level-1 codebook C1 [256][d] once per CTA, then one
 // region per warp.
 struct WalkSmem {
-    size_t yq, stage, wkey, wflag, cand, cunsorted, slot, rowbuf, hash, total;
+    size_t yq, stage, wkey, cand, sel, slot, hash, total;
 };
 
 // Layout of the walk's level-1 codebook in shared memory, chosen so that a lane's sub-space
@@ -117,13 +158,11 @@ struct WalkSmem {
 //  0 (row-major): row c holds centroid c of every sub-space in its own coordinates ([256][d]).
 //    Used in FP32 with 3 or 6 dimensions per sub-space (3 j + u mod 32 permutes the lanes)
 //    and for non-uniform splits.
-//  1 (interleaved): the P values (D1 rounded up to 2 or 8) of centroid c in sub-space j sit
-//    at (c * M1 + j) * P: one vector load.  FP32 and FP16 with 2 dimensions, FP16 with 6.
-//  2 (split, FP16 with 3 dimensions): the first two values as a half2 array [256][M1], the
-//    third as a half array [256][M1] behind it: two loads, no padding.
+//  1 (interleaved): the P values (D1 rounded up to 2, 4 or 8) of centroid c in sub-space j sit
+//    at (c * M1 + j) * P: one vector load.  FP32 and FP16 with 2 dimensions, FP16 with 3 and 6.
 __host__ __device__ constexpr int walk_layout(int D1, int es)
 {
-    return D1 == 0 ? 0 : D1 == 2 ? 1 : es == 4 ? 0 : D1 == 3 ? 2 : 1;
+    return D1 == 0 ? 0 : D1 == 2 ? 1 : es == 4 ? 0 : 1;
 }
 __host__ __device__ constexpr int walk_pad(int D1) { return D1 <= 2 ? 2 : (D1 <= 4 ? 4 : 8); }
 // bytes of the level-1 codebook in shared memory (es = 4: FP32, es = 2: FP16)
@@ -133,11 +172,19 @@ __host__ __device__ inline size_t walk_c1_bytes(int d, int M1, int D1, size_t es
     const size_t n = L == 1 ? (size_t)256 * M1 * walk_pad(D1) : (size_t)256 * d;
     return align_up(n * es, 128);
 }
+// Layout of the full walk's FP16 level-2 codebook in shared memory: with 3 dimensions per
+// level-1 sub-space as the level-1 codebook's layout 1 (the values of a lane's coordinates, for
+// every centroid: one 8-byte load), else row-major [256][d].  The FP32 one is row-major.
+__host__ __device__ constexpr bool walk_c2_lanes(int D1, int es) { return D1 == 3 && es == 2; }
+__host__ __device__ inline size_t walk_c2_bytes(int d, int M1, int D1)
+{
+    return align_up((walk_c2_lanes(D1, 2) ? (size_t)256 * M1 * walk_pad(D1) : (size_t)256 * d) * 2, 128);
+}
 // shared memory before the per-warp regions: the walk's level-1 codebook and, for the full
-// walk in FP16, C2 [256][d] behind it
+// walk in FP16, the level-2 codebook behind it
 __host__ __device__ inline size_t walk_cb_bytes(int d, int M1, int D1, size_t es, bool fq)
 {
-    return walk_c1_bytes(d, M1, D1, es) + (fq && es == 2 ? align_up((size_t)256 * d * 2, 128) : 0);
+    return walk_c1_bytes(d, M1, D1, es) + (fq && es == 2 ? walk_c2_bytes(d, M1, D1) : 0);
 }
 // compile-time sub-space width of the uniform splits 96/16, 96/32 and 128/64 (0: other)
 __host__ __device__ constexpr int walk_variant_d1(int variant) { return variant == 1 ? 6 : variant == 2 ? 3 : variant == 3 ? 2 : 0; }
@@ -149,29 +196,53 @@ inline int walk_variant(int M1, int d)
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__half x) { return __half2float(x); }
 
+// Nodes whose code rows are staged together: two chunks of 32 where a step can have that many
+// fresh nodes (beam > 1) and a row is at most 32 bytes, so that most steps wait for global memory
+// once; one chunk otherwise (a second one would cost walks in flight).
+__host__ __device__ constexpr int stage_rows(int row_bytes, int beam, int tag)
+{
+    return tag && beam > 1 && row_bytes <= 32 ? 64 : 32;
+}
 // own_rot: the walk rotates the query itself (y' in shared memory); otherwise y' is read from
-// the rotation kernel's output.  Areas whose lives do not overlap within a step share memory:
-// the adjacency rows are read before the candidates are collected (the unsorted-candidate
-// area), and the staged code rows are dead once the step's nodes are scored, before the
-// candidates are sorted (the sorted-candidate area).  W is one buffer, merged in place.
-__host__ __device__ inline WalkSmem walk_smem(int M1, int d, int efcap, int hash_log, int beam, bool own_rot,
+// the rotation kernel's output.
+__host__ __device__ inline WalkSmem walk_smem(int M1, int d, int efcap, const VisitTab &vt, int beam, bool own_rot,
                                              int m2p = 0)
 {
     WalkSmem s;
     size_t o = 0;
     s.yq = o;        o += own_rot ? align_up((size_t)d * 4, 16) : 0;
-    s.stage = o;                                       // level-1 rows, then (full walk) residual rows
-    const size_t st_b = (size_t)32 * (M1 + m2p), cd_b = (size_t)32 * beam * 8;
-    s.cand = o;      o += align_up(st_b > cd_b ? st_b : cd_b, 16);
+    s.stage = o;     o += (size_t)stage_rows(M1 + m2p, beam, vt.tag) * (M1 + m2p);   // level-1 rows, then residual rows
     s.wkey = o;      o += (size_t)efcap * 8;
-    s.wflag = o;     o += align_up((size_t)efcap, 16);
-    s.cunsorted = o; o += (size_t)32 * beam * 8;
-    s.rowbuf = s.cunsorted;
+    s.cand = o;      o += (size_t)32 * beam * 8 + 32;                          // candidates of a step, padded
+    s.sel = o;       o += 32;                                                // nodes expanded in a step (at most 8)
     s.slot = o;      o += (size_t)32 * beam * 4;
-    s.hash = o;      o += ((size_t)1 << hash_log) * 4;
+    s.hash = o;      o += visit_bytes(vt);
     s.total = align_up(o, 128);
     return s;
 }
+// The size by which a search too wide for the shared memory is refused: a walk with a table of
+// 32-bit ids of its limits' size, next to codebooks without padding (so that what is accepted does
+// not depend on how the walk lays out its memory).
+inline size_t walk_nominal_cb_bytes(int d, int M1, bool half, bool full)
+{
+    const int D1 = walk_variant_d1(walk_variant(M1, d));
+    const size_t plain = align_up((size_t)256 * d * 2, 128);
+    return (half && D1 == 3 ? plain : walk_c1_bytes(d, M1, D1, half ? 2 : 4)) + (full && half ? plain : 0);
+}
+inline size_t walk_smem_nominal(int M1, int d, int efcap, int hash_log, int beam, bool own_rot, int m2p = 0)
+{
+    const size_t st_b = (size_t)32 * (M1 + m2p), cd_b = (size_t)32 * beam * 8;
+    return align_up((own_rot ? align_up((size_t)d * 4, 16) : 0) + align_up(std::max(st_b, cd_b), 16) + (size_t)efcap * 8 +
+                        align_up((size_t)efcap, 16) + (size_t)32 * beam * 12 + ((size_t)4 << hash_log), 128);
+}
+
+// Keys of the result list: distance bits, id, and the "expanded" flag as the lowest bit, which
+// never decides an order (ids are distinct).
+__device__ __forceinline__ uint64_t walk_key(float dist, int32_t id)
+{
+    return ((uint64_t)__float_as_uint(dist) << 32) | ((uint32_t)id << 1);
+}
+__device__ __forceinline__ int32_t walk_id(uint64_t k) { return (int32_t)((uint32_t)k >> 1); }
 
 __device__ __forceinline__ uint64_t make_key(float dist, int32_t id)
 {
@@ -180,54 +251,18 @@ __device__ __forceinline__ uint64_t make_key(float dist, int32_t id)
 __device__ __forceinline__ int32_t key_id(uint64_t k) { return (int32_t)(uint32_t)(k & 0xffffffffu); }
 __device__ __forceinline__ float key_dist(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
 
-__device__ __forceinline__ uint64_t shfl_xor64(uint64_t v, int m)
+// Smallest (distance, id) of the lanes' pairs (distance bits ~0: none), by two warp reductions.
+__device__ __forceinline__ void warp_best(uint32_t dist, uint32_t id, uint32_t *bd, uint32_t *bi)
 {
-    uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
-    lo = __shfl_xor_sync(FULL, lo, m);
-    hi = __shfl_xor_sync(FULL, hi, m);
-    return ((uint64_t)hi << 32) | lo;
-}
-
-__device__ __forceinline__ uint64_t warp_min64(uint64_t v)
-{
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
-        uint64_t o = shfl_xor64(v, m);
-        v = o < v ? o : v;
-    }
-    return v;
+    *bd = __reduce_min_sync(0xffffffffu, dist);
+    *bi = __reduce_min_sync(0xffffffffu, dist == *bd ? id : 0xffffffffu);
 }
 
 // Lane bits in the order partial distances are combined: 3, 2, 1, 0, then 4.
 __host__ __device__ constexpr int comb_bit(int k) { return k < 4 ? 3 - k : 4; }
 __host__ __device__ constexpr int ilog2c(int s) { return s <= 1 ? 0 : 1 + ilog2c(s >> 1); }
 
-// Sum over the 32 lanes of S per-slot contributions (S a power of two): reduce-scatter along
-// the first log2(S) combination bits, all-reduce along the rest.  The addition tree of
-// every slot is the same (lanes differing in bit 3 first, then 2, 1, 0, 4), whatever S.
-template <int S>
-__device__ __forceinline__ float reduce_slots(float (&v)[S], int lane)
-{
-    constexpr int LS = ilog2c(S);
-#pragma unroll
-    for (int k = 0; k < LS; k++) {
-        const int bit = comb_bit(k);
-        const int half = (S >> k) >> 1;
-        const bool hi = (lane >> bit) & 1;
-#pragma unroll
-        for (int i = 0; i < half; i++) {
-            float send = hi ? v[i] : v[i + half];
-            float keep = hi ? v[i + half] : v[i];
-            v[i] = keep + __shfl_xor_sync(FULL, send, 1 << bit);
-        }
-    }
-    float r = v[0];
-#pragma unroll
-    for (int k = LS; k < 5; k++) r += __shfl_xor_sync(FULL, r, 1 << comb_bit(k));
-    return r;
-}
-
-// Slot whose total lane `lane` holds after reduce_slots<S> (S = 2^LS).
+// The lane bits of the first LS combinations, the first one most significant.
 __device__ __forceinline__ int slot_of_lane(int lane, int LS)
 {
     int s = 0;
@@ -243,9 +278,44 @@ template <int M1, int D1>
 struct LaneGeo {
     static constexpr int NSUB = M1 == 64 ? 2 : 1;
     static constexpr int DMAX = D1 > 0 ? D1 : (M1 == 16 ? 16 : (M1 == 32 ? 8 : 4));   // d <= 256
+    static constexpr int M2W = (DMAX + 3) / 4;
     int off[NSUB], len[NSUB], j[NSUB];
+    int maxlen;                  // longest sub-space (D1 = 0)
     float y[NSUB][DMAX];
-    int m2[NSUB][DMAX];          // full walk: level-2 sub-space of each of the lane's coordinates
+    // full walk: the level-2 sub-space of each of the lane's coordinates, four per word, and
+    // whether no lane's coordinates touch more than two (warp-uniform)
+    uint32_t m2[NSUB][M2W];
+    bool two;
+
+    __device__ __forceinline__ int sub2(int k, int u) const { return (m2[k][u / 4] >> (8 * (u % 4))) & 0xff; }
+
+    __device__ __forceinline__ void init(const SplitTab &s1, const float *yrot, const uint8_t *sub2tab, int d, int lane)
+    {
+        two = true;
+        maxlen = D1 > 0 ? D1 : (d + M1 - 1) / M1;
+#pragma unroll
+        for (int k = 0; k < NSUB; k++) {
+            const int jj = M1 == 16 ? (lane & 15) : lane + 32 * k;
+            j[k] = jj;
+            off[k] = D1 > 0 ? D1 * jj : s1.off[jj];
+            len[k] = D1 > 0 ? D1 : s1.len[jj];
+#pragma unroll
+            for (int u = 0; u < DMAX; u++) y[k][u] = D1 > 0 || u < len[k] ? yrot[off[k] + u] : 0.f;
+            if (sub2tab) {
+#pragma unroll
+                for (int w = 0; w < M2W; w++) m2[k][w] = 0;
+#pragma unroll
+                for (int u = 0; u < DMAX; u++)
+                    if (D1 > 0 || u < len[k]) m2[k][u / 4] |= (uint32_t)sub2tab[off[k] + u] << (8 * (u % 4));
+                if (D1 > 2) {
+#pragma unroll
+                    for (int u = 1; u < D1 - 1; u++)
+                        two = two && (sub2(k, u) == sub2(k, 0) || sub2(k, u) == sub2(k, D1 - 1));
+                }
+            }
+        }
+        if (D1 > 2) two = __all_sync(FULL, two);
+    }
 };
 
 __device__ __forceinline__ void half2_to_f(uint32_t w, float &a, float &b)
@@ -262,11 +332,7 @@ __device__ __forceinline__ void load_row(const CT *C1s, int d, int c, const Lane
 {
     constexpr int DMAX = LaneGeo<M1, D1>::DMAX;
     constexpr int LAYOUT = walk_layout(D1, (int)sizeof(CT));
-    if constexpr (LAYOUT == 2) {
-        const uint32_t w = *reinterpret_cast<const uint32_t *>(C1s + ((size_t)c * M1 + g.j[k]) * 2);
-        half2_to_f(w, x[0], x[1]);
-        x[2] = to_f(C1s[(size_t)256 * M1 * 2 + (size_t)c * M1 + g.j[k]]);
-    } else if constexpr (LAYOUT == 1) {
+    if constexpr (LAYOUT == 1) {
         constexpr int P = walk_pad(D1);
         const CT *p = C1s + ((size_t)c * M1 + g.j[k]) * P;
         float t[P];
@@ -276,6 +342,10 @@ __device__ __forceinline__ void load_row(const CT *C1s, int d, int c, const Lane
             t[1] = f.y;
         } else if constexpr (P == 2) {
             half2_to_f(*reinterpret_cast<const uint32_t *>(p), t[0], t[1]);
+        } else if constexpr (P == 4) {
+            const uint2 w = *reinterpret_cast<const uint2 *>(p);
+            half2_to_f(w.x, t[0], t[1]);
+            half2_to_f(w.y, t[2], t[3]);
         } else {
             const uint4 w = *reinterpret_cast<const uint4 *>(p);
             half2_to_f(w.x, t[0], t[1]);
@@ -288,32 +358,9 @@ __device__ __forceinline__ void load_row(const CT *C1s, int d, int c, const Lane
     } else {
         const CT *row = C1s + c * d + g.off[k];
 #pragma unroll
-        for (int u = 0; u < DMAX; u++) x[u] = (D1 > 0 || u < g.len[k]) ? to_f(row[u]) : 0.f;
+        for (int u = 0; u < DMAX; u++)
+            if (D1 > 0 || u < g.maxlen) x[u] = (D1 > 0 || u < g.len[k]) ? to_f(row[u]) : 0.f;
     }
-}
-
-// ||y'^j - C1_j[c]||^2 in the fixed order of the sub-space's coordinates.
-template <int M1, int D1, typename CT>
-__device__ __forceinline__ float part_dist(const CT *C1s, int d, int c, const LaneGeo<M1, D1> &g, int k)
-{
-    float x[LaneGeo<M1, D1>::DMAX];
-    load_row<M1, D1, CT>(C1s, d, c, g, k, x);
-    float s = 0.f;
-    if (D1 > 0) {
-#pragma unroll
-        for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++) {
-            float df = g.y[k][u] - x[u];
-            s = fmaf(df, df, s);
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++)
-            if (u < g.len[k]) {
-                float df = g.y[k][u] - x[u];
-                s = fmaf(df, df, s);
-            }
-    }
-    return s;
 }
 
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi)
@@ -329,8 +376,8 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float &lo, float &
 }
 
 // The sub-space terms of two codes c0, c1 at once with packed FP32x2 arithmetic: each half
-// performs exactly the scalar operations of part_dist (same rounding), two slots per
-// instruction.
+// performs the scalar operations in the order of the sub-space's coordinates (same rounding),
+// two slots per instruction.
 template <int M1, int D1, typename CT>
 __device__ __forceinline__ void pair_dist(const CT *C1s, int d, int c0, int c1, const LaneGeo<M1, D1> &g,
                                           int k, float &s0, float &s1)
@@ -355,133 +402,242 @@ __device__ __forceinline__ void pair_dist(const CT *C1s, int d, int c0, int c1, 
 __device__ __forceinline__ float c2_at(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float c2_at(const __half *p) { return __half2float(*p); }
 
-// Full walk: sum over this lane's coordinates t of (y'_t - (C1[c1][t] + C2[c2_m(t)][t]))^2,
-// where row2 is the node's staged residual row and m(t) the level-2 sub-space of t.
-template <int M1, int D1, typename CT>
-__device__ __forceinline__ float part_full(const CT *C1s, const CT *C2, int d, int c, const uint8_t *row2,
-                                           const LaneGeo<M1, D1> &g, int k)
+// The level-2 values of this lane's coordinates for a node whose staged residual row is row2.
+// At most two level-2 sub-spaces per lane (TWO): the first and the last coordinate's code, each
+// coordinate taking the one of its sub-space; else a code per coordinate.
+template <int M1, int D1, typename CT, bool TWO>
+__device__ __forceinline__ void load_row2(const CT *C2, int d, const uint8_t *row2, const LaneGeo<M1, D1> &g, int k,
+                                          float (&z)[LaneGeo<M1, D1>::DMAX])
 {
-    float x[LaneGeo<M1, D1>::DMAX];
-    load_row<M1, D1, CT>(C1s, d, c, g, k, x);
-    float s = 0.f;
+    constexpr int DMAX = LaneGeo<M1, D1>::DMAX;
+    if constexpr (walk_c2_lanes(D1, (int)sizeof(CT))) {
+        auto at = [&](int c) { return *reinterpret_cast<const uint2 *>(C2 + ((size_t)c * M1 + g.j[k]) * 4); };
+        const uint2 wa = at(row2[g.sub2(k, 0)]), wb = at(row2[g.sub2(k, 2)]);
+        // coordinates 0 and 1 share a word, as do 2 and the padding
+        float t;
+        half2_to_f(wa.x, z[0], t);
+        half2_to_f(wb.y, z[2], t);
+        if (TWO) half2_to_f(g.sub2(k, 1) == g.sub2(k, 0) ? wa.x : wb.x, t, z[1]);
+        else half2_to_f(at(row2[g.sub2(k, 1)]).x, t, z[1]);
+    } else if constexpr (TWO && D1 > 0) {
+        const int ca = row2[g.sub2(k, 0)], cb = row2[g.sub2(k, D1 - 1)];
+        const CT *pa = C2 + (size_t)ca * d + g.off[k], *pb = C2 + (size_t)cb * d + g.off[k];
 #pragma unroll
-    for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++) {
-        if (D1 == 0 && u >= g.len[k]) continue;
-        const float v = x[u] + c2_at(C2 + (int)row2[g.m2[k][u]] * d + g.off[k] + u);
-        const float df = g.y[k][u] - v;
-        s = fmaf(df, df, s);
+        for (int u = 0; u < D1; u++) z[u] = c2_at((g.sub2(k, u) == g.sub2(k, 0) ? pa : pb) + u);
+    } else {
+#pragma unroll
+        for (int u = 0; u < DMAX; u++)
+            z[u] = D1 > 0 || u < g.len[k] ? c2_at(C2 + (size_t)row2[g.sub2(k, u)] * d + g.off[k] + u) : 0.f;
     }
-    return s;
 }
 
-// Sub-space terms of S slots (S = 16 or 32) for this lane, summed by reduce_slots<S>.  TAB:
-// C1s is the query's ADC table [256][M1] (FP16) and the term of code c is its entry [c][lane].
-template <int M1, int D1, int S, typename CT, bool FQ, bool TAB = false>
-__device__ __forceinline__ float score_slots(const CT *C1s, const uint8_t *stage, int nf, int d,
-                                             const LaneGeo<M1, D1> &g, int lane, const CT *C2, int M2P)
+// Full walk, two nodes at once: sums over this lane's coordinates t of
+// (y'_t - (C1[c1][t] + C2[c2_m(t)][t]))^2 in the order of the coordinates, m(t) the level-2
+// sub-space of t, in packed FP32 arithmetic (the scalar operations' roundings).
+template <int M1, int D1, typename CT, bool TWO>
+__device__ __forceinline__ void pair_full(const CT *C1s, const CT *C2, int d, int c0, int c1, const uint8_t *ra,
+                                          const uint8_t *rb, const LaneGeo<M1, D1> &g, int k, float &s0, float &s1)
 {
-    float v[S];
+    constexpr int DMAX = LaneGeo<M1, D1>::DMAX;
+    float x0[DMAX], x1[DMAX], z0[DMAX], z1[DMAX];
+    load_row<M1, D1, CT>(C1s, d, c0, g, k, x0);
+    load_row<M1, D1, CT>(C1s, d, c1, g, k, x1);
+    load_row2<M1, D1, CT, TWO>(C2, d, ra, g, k, z0);
+    load_row2<M1, D1, CT, TWO>(C2, d, rb, g, k, z1);
+    unsigned long long acc = 0ull;
+#pragma unroll
+    for (int u = 0; u < DMAX; u++) {
+        if (D1 == 0 && u >= g.maxlen) continue;
+        const unsigned long long yy = pack2(g.y[k][u], g.y[k][u]);
+        unsigned long long v, df;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pack2(x0[u], x1[u])), "l"(pack2(z0[u], z1[u])));
+        asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(df) : "l"(yy), "l"(v));
+        asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(acc) : "l"(df), "l"(acc));
+    }
+    unpack2(acc, s0, s1);
+}
+
+// Scoring works on blocks of slot_block staged nodes, eight values per lane, summed over the
+// lanes differing in bits 3, 2 and 1 by a reduce-scatter (seven shuffles), then over bit 0 and,
+// with 32 sub-space lanes, bit 4 (one total left per lane).  With M1 = 16 the two half-warps
+// score different nodes, so a block has 16.  Lane order: with s3 = the lane's bits 3, 2, 1 (bit
+// 3 first), value i of a lane belongs to node i ^ s3, so at each level every lane keeps its
+// lower half and sends its upper one, without selects, and ends with node s3.  A lane keeps
+// the total of one node per chunk of 32: node chunk_slot(lane).
+// Blocks of eight in a rolled loop, and not one unrolled pass over 16 or 32 nodes: fewer
+// registers (24 warps per SM leave 80 each), no work past the last block, and code that stays in
+// the instruction cache (the unrolled full-decode scoring lost two thirds of its stall cycles
+// waiting for instructions).
+__host__ __device__ constexpr int slot_block(int M1) { return M1 == 16 ? 16 : 8; }
+
+template <int M1>
+__device__ __forceinline__ int lane_block(int lane)
+{
+    return M1 == 16 ? (lane & 1) : ((lane & 1) | ((lane >> 3) & 2));
+}
+
+template <int M1>
+__device__ __forceinline__ int chunk_slot(int lane)
+{
+    const int s3 = slot_of_lane(lane, 3);
+    return lane_block<M1>(lane) * slot_block(M1) + (M1 == 16 ? 2 * s3 + (lane >> 4) : s3);
+}
+
+// The eight values of this lane for the block staged at `stage` (residual rows at `stage2`).
+// Slots past the nodes staged hold stale bytes, which are codes all the same; their totals are
+// not used.  TAB: C1s is the query's ADC table [256][M1] (FP16): the term of code c is its entry
+// [c][lane].
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool TWO>
+__device__ __forceinline__ void block_terms(const CT *C1s, const uint8_t *stage, const uint8_t *stage2, int d,
+                                            const LaneGeo<M1, D1> &g, int lane, const CT *C2, int M2P, float (&v)[8])
+{
+    // node of value i for this lane, and its code in sub-space j
+    const int h = M1 == 16 ? lane >> 4 : 0, j = M1 == 16 ? lane & 15 : lane, s3 = slot_of_lane(lane, 3);
+    auto slot = [&](int i) { return M1 == 16 ? 2 * (i ^ s3) + h : i ^ s3; };
     if constexpr (TAB) {
         static_assert(M1 == 32 && !FQ, "the table form is built for 32 sub-spaces");
 #pragma unroll
-        for (int i = 0; i < S; i++) v[i] = i < nf ? to_f(C1s[(int)stage[i * M1 + lane] * M1 + lane]) : 0.f;
+        for (int i = 0; i < 8; i++) v[i] = to_f(C1s[(int)stage[slot(i) * M1 + lane] * M1 + lane]);
     } else if constexpr (FQ) {
-        // full walk: one slot per step; the residual rows follow the 32 level-1 rows
-        const uint8_t *stage2 = stage + 32 * M1;
-        if (M1 == 16) {
-            const int h = lane >> 4, j = lane & 15;
 #pragma unroll
-            for (int i = 0; i < S / 2; i++) {
-                const int sl = 2 * i + h;
-                float t = 0.f;
-                if (2 * i < nf && sl < nf) t = part_full<M1, D1, CT>(C1s, C2, d, stage[sl * 16 + j], stage2 + sl * M2P, g, 0);
-                v[2 * i] = h ? 0.f : t;
-                v[2 * i + 1] = h ? t : 0.f;
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < S; i++) {
-                float t = 0.f;
-                if (i < nf) {
-                    t = part_full<M1, D1, CT>(C1s, C2, d, stage[i * M1 + lane], stage2 + i * M2P, g, 0);
-                    if (M1 == 64) t += part_full<M1, D1, CT>(C1s, C2, d, stage[i * M1 + 32 + lane], stage2 + i * M2P, g, 1);
-                }
-                v[i] = t;
+        for (int i = 0; i < 8; i += 2) {
+            const uint8_t *ca = stage + slot(i) * M1, *cb = stage + slot(i + 1) * M1;
+            const uint8_t *ra = stage2 + slot(i) * M2P, *rb = stage2 + slot(i + 1) * M2P;
+            pair_full<M1, D1, CT, TWO>(C1s, C2, d, ca[j], cb[j], ra, rb, g, 0, v[i], v[i + 1]);
+            if (M1 == 64) {
+                float u0, u1;
+                pair_full<M1, D1, CT, TWO>(C1s, C2, d, ca[32 + j], cb[32 + j], ra, rb, g, LaneGeo<M1, D1>::NSUB - 1, u0, u1);
+                v[i] += u0;
+                v[i + 1] += u1;
             }
         }
-    } else if (M1 == 16) {
-        const int h = lane >> 4, j = lane & 15;
+    } else if constexpr (D1 > 0) {
 #pragma unroll
-        for (int i = 0; i < S / 2; i++) {
-            const int sl = 2 * i + h;                // half-warp h scores slots of parity h
-            float t = 0.f;
-            if (2 * i < nf && sl < nf) t = part_dist<M1, D1, CT>(C1s, d, stage[sl * 16 + j], g, 0);
-            v[2 * i] = h ? 0.f : t;
-            v[2 * i + 1] = h ? t : 0.f;
-        }
-    } else if (D1 > 0) {
-        // two slots per step (the staged row of slot i + 1 >= nf is stale but a valid code;
-        // its term is discarded)
-#pragma unroll
-        for (int i = 0; i < S; i += 2) {
-            float t0 = 0.f, t1 = 0.f;
-            if (i < nf) {
-                pair_dist<M1, D1, CT>(C1s, d, stage[i * M1 + lane], stage[(i + 1) * M1 + lane], g, 0, t0, t1);
-                if (M1 == 64) {
-                    float u0, u1;
-                    pair_dist<M1, D1, CT>(C1s, d, stage[i * M1 + 32 + lane], stage[(i + 1) * M1 + 32 + lane], g, 1, u0, u1);
-                    t0 += u0;
-                    t1 += u1;
-                }
-                if (i + 1 >= nf) t1 = 0.f;
+        for (int i = 0; i < 8; i += 2) {
+            const uint8_t *ca = stage + slot(i) * M1, *cb = stage + slot(i + 1) * M1;
+            pair_dist<M1, D1, CT>(C1s, d, ca[j], cb[j], g, 0, v[i], v[i + 1]);
+            if (M1 == 64) {
+                float u0, u1;
+                pair_dist<M1, D1, CT>(C1s, d, ca[32 + j], cb[32 + j], g, LaneGeo<M1, D1>::NSUB - 1, u0, u1);
+                v[i] += u0;
+                v[i + 1] += u1;
             }
-            v[i] = t0;
-            v[i + 1] = t1;
         }
     } else {
+        // uneven split: coordinate by coordinate over the eight nodes; those past a lane's own
+        // length count 0 (fma(0, 0, s) = s)
 #pragma unroll
-        for (int i = 0; i < S; i++) {
-            float t = 0.f;
-            if (i < nf) {
-                t = part_dist<M1, D1, CT>(C1s, d, stage[i * M1 + lane], g, 0);
-                if (M1 == 64) t += part_dist<M1, D1, CT>(C1s, d, stage[i * M1 + 32 + lane], g, 1);
+        for (int k = 0; k < LaneGeo<M1, D1>::NSUB; k++) {
+            const CT *row[8];
+            float t[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                row[i] = C1s + (int)stage[slot(i) * M1 + 32 * k + j] * d + g.off[k];
+                t[i] = 0.f;
             }
-            v[i] = t;
+#pragma unroll
+            for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++) {
+                if (u >= g.maxlen) break;
+                const bool in = u < g.len[k];
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    const float df = in ? g.y[k][u] - to_f(row[i][in ? u : 0]) : 0.f;
+                    t[i] = fmaf(df, df, t[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; i++) v[i] = k ? v[i] + t[i] : t[i];
         }
     }
-    return reduce_slots<S>(v, lane);
 }
 
-// Walk distances of the nf nodes in slot[0..nf) (1 <= nf <= 32): their code rows are staged
-// in shared memory, each lane computes its sub-space terms, and the totals are formed with
-// 16 or 32 slots.  Returns lane's total; *my_slot = the slot it holds (>= 32: none).
-template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
-__device__ __forceinline__ float score_nodes(const CT *C1s, uint8_t *stage, const uint8_t *codes1,
-                                             const int32_t *slot, int nf, int d,
-                                             const LaneGeo<M1, D1> &g, int lane, int *my_slot,
-                                             const CT *C2, const uint8_t *codes2b, int M2P)
+// Sum of a block's eight values over the sub-space lanes, in the fixed order (bits 3, 2, 1, 0,
+// then 4); with M1 = 16 the half-warps hold different nodes (bit 4 would add their zeros).
+template <int M1>
+__device__ __forceinline__ float reduce_block(float (&v)[8])
 {
-    if (lane < nf) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(codes1 + (int64_t)slot[lane] * M1);
-        uint4 *dst = reinterpret_cast<uint4 *>(stage + lane * M1);
 #pragma unroll
-        for (int u = 0; u < M1 / 16; u++) dst[u] = __ldg(src + u);
-        if constexpr (FQ) {
-            const uint4 *s2 = reinterpret_cast<const uint4 *>(codes2b + (int64_t)slot[lane] * M2P);
-            uint4 *d2 = reinterpret_cast<uint4 *>(stage + 32 * M1 + lane * M2P);
-            for (int u = 0; u < M2P / 16; u++) d2[u] = __ldg(s2 + u);
+    for (int k = 0; k < 3; k++) {
+        const int half = 4 >> k;
+#pragma unroll
+        for (int i = 0; i < half; i++) v[i] += __shfl_xor_sync(FULL, v[i + half], 1 << comb_bit(k));
+    }
+    float r = v[0];
+    r += __shfl_xor_sync(FULL, r, 1);
+    if (M1 != 16) r += __shfl_xor_sync(FULL, r, 16);
+    return r;
+}
+
+// Copies bytes (a multiple of 16) into shared memory with every load of a thread in flight at
+// once (cp.async), so a block of a single warp does not wait for each; copy_wait before a
+// barrier.
+__device__ __forceinline__ void copy16(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void copy_async(void *dst, const void *src, size_t bytes)
+{
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x * 16; i < bytes; i += blockDim.x * 16)
+        copy16(static_cast<char *>(dst) + i, static_cast<const char *>(src) + i);
+}
+
+// Code rows of the n nodes in slot[0..n) (n <= rows) into the staging area: the level-1 rows,
+// then, for the full walk, the residual rows behind all `rows` of them.
+template <int M1, bool FQ>
+__device__ __forceinline__ void stage_codes(uint8_t *stage, int rows, const uint8_t *codes1, const uint8_t *codes2b, int M2P,
+                                            const int32_t *slot, int n, int lane)
+{
+    __syncwarp();                                        // slot written, the staged rows read
+#pragma unroll
+    for (int i0 = 0; i0 < 64; i0 += 32) {
+        if (i0 >= n) break;
+        const int i = i0 + lane;
+        if (i < n) {
+            const int64_t v = slot[i];
+#pragma unroll
+            for (int u = 0; u < M1 / 16; u++) copy16(stage + i * M1 + 16 * u, codes1 + v * M1 + 16 * u);
+            if constexpr (FQ)
+                for (int u = 0; u < M2P; u += 16) copy16(stage + rows * M1 + i * M2P + u, codes2b + v * M2P + u);
         }
     }
+    copy_wait();
     __syncwarp();
-    float r;
-    if (nf <= 16) {
-        r = score_slots<M1, D1, 16, CT, FQ, TAB>(C1s, stage, nf, d, g, lane, C2, M2P);
-        *my_slot = lane < 16 ? lane : 32;           // lanes l and l + 16 hold slot l
-    } else {
-        r = score_slots<M1, D1, 32, CT, FQ, TAB>(C1s, stage, nf, d, g, lane, C2, M2P);
-        *my_slot = slot_of_lane(lane, 5);
+}
+
+// Walk distances of nf staged nodes (1 <= nf <= 32), block by block, two blocks at once where
+// there are two (their chains of shared-memory reads and shuffles overlap).  Returns the total of
+// node chunk_slot(lane) (undefined from nf on).
+template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
+__device__ __forceinline__ float score_staged(const CT *C1s, const uint8_t *stage, const uint8_t *stage2, int nf, int d,
+                                              const LaneGeo<M1, D1> &g, int lane, const CT *C2, int M2P)
+{
+    constexpr int SB = slot_block(M1);
+    const int mine = lane_block<M1>(lane);
+    float r = 0.f;
+    auto terms = [&](int b, float (&v)[8]) {
+        const uint8_t *st = stage + b * SB * M1, *st2 = stage2 + b * SB * M2P;
+        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, TAB, false>(C1s, st, st2, d, g, lane, C2, M2P, v);
+        else block_terms<M1, D1, CT, FQ, TAB, true>(C1s, st, st2, d, g, lane, C2, M2P, v);
+    };
+    constexpr bool PAIR = !FQ && D1 > 0;
+#pragma unroll 1
+    for (int b = 0; b * SB < nf; b += PAIR ? 2 : 1) {
+        float v[8];
+        if (PAIR && (b + 1) * SB < nf) {
+            float v1[8];
+            terms(b, v);
+            terms(b + 1, v1);
+            const float t = reduce_block<M1>(v), t1 = reduce_block<M1>(v1);
+            if (b == mine) r = t;
+            if (b + 1 == mine) r = t1;
+        } else {
+            terms(b, v);
+            const float t = reduce_block<M1>(v);
+            if (b == mine) r = t;
+        }
     }
-    __syncwarp();
     return r;
 }
 
@@ -491,95 +647,396 @@ __device__ __forceinline__ uint32_t hash32(int32_t e)
     return x ^ (x >> 15);
 }
 
-// Open addressing with triangular probing: the p-th probe of id e is at hash(e) + p(p+1)/2
-// (mod the power-of-two table size), which visits every slot and, unlike a linear probe, does
-// not grow long runs of occupied slots as the table fills (a warp resolves a row of 32 ids
-// only when its longest probe sequence ends).
-// Inserts e into the visited set; true if it was not there.  The shared table takes
-// inserts until the walk switches to spill mode; from then on it is only read and new ids
-// go to the warp's global table.
-// Ids the shared visited table of H entries takes before the walk switches to the global one.
-// Filling to three quarters rather than half (triangular probing: probe sequences stay short)
-// measured 0.606 against 0.645 ms for the 1M workload's level-0 launch (fewer walks spill);
-// seven eighths measured 0.654 ms.
+// Ids counted to the shared part of the visited set before the walk counts to the global one.
 __host__ __device__ constexpr int shared_visited_cap(int H) { return H - H / 4; }
 
-__device__ __forceinline__ bool visit(int32_t e, int32_t *hash, int hlog, bool spilled,
-                                      int32_t *spill, int slog)
+// Open addressing with triangular probing (the p-th probe of id e at hash(e) + p(p+1)/2, mod the
+// power-of-two size, visits every entry), -1 = empty.  table_insert: true if e was not there.
+__device__ __forceinline__ bool table_insert(int32_t e, int32_t *tab, int log, int shift)
 {
-    uint32_t Hm = (1u << hlog) - 1;
-    uint32_t h = hash32(e) & Hm;
-    if (!spilled) {
-        for (uint32_t p = 0; p <= Hm; p++) {
-            int32_t old = atomicCAS(hash + h, -1, e);
-            if (old == -1) return true;
-            if (old == e) return false;
-            h = (h + p + 1) & Hm;
-        }
-        return false;   // unreachable: the table is kept at most three quarters full
-    }
-    for (uint32_t p = 0; p <= Hm; p++) {
-        int32_t v = hash[h];
-        if (v == e) return false;
-        if (v == -1) break;
-        h = (h + p + 1) & Hm;
-    }
-    uint32_t Sm = (1u << slog) - 1;
-    h = (hash32(e) >> 3) & Sm;
-    for (uint32_t p = 0; p <= Sm; p++) {
-        int32_t old = atomicCAS(spill + h, -1, e);
+    const uint32_t m = (1u << log) - 1;
+    uint32_t h = (hash32(e) >> shift) & m;
+#pragma unroll 1
+    for (uint32_t p = 0; p <= m; p++) {
+        const int32_t old = atomicCAS(tab + h, -1, e);
         if (old == -1) return true;
         if (old == e) return false;
-        h = (h + p + 1) & Sm;
+        h = (h + p + 1) & m;
     }
-    return false;       // unreachable: the spill table is kept at most half full
+    return false;                  // unreachable: the table is never full
+}
+__device__ __forceinline__ bool table_find(int32_t e, const int32_t *tab, int log, int shift)
+{
+    const uint32_t m = (1u << log) - 1;
+    uint32_t h = (hash32(e) >> shift) & m;
+#pragma unroll 1
+    for (uint32_t p = 0; p <= m; p++) {
+        const int32_t v = tab[h];
+        if (v == e) return true;
+        if (v == -1) return false;
+        h = (h + p + 1) & m;
+    }
+    return false;
+}
+
+// A halfword of v that is zero, as a mask with bit 15 or 31 set; exact for "is there one", and
+// for which ones when the zero halfwords are the high ones of the word (as empty entries are:
+// a bucket fills from its first entry on).
+__device__ __forceinline__ uint32_t zero16(uint32_t v) { return (v - 0x00010001u) & ~v & 0x80008000u; }
+
+// Shared-memory accesses by 32-bit address.
+__device__ __forceinline__ uint4 lds128(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+// One look at the bucket of id e (e < 0: no id): SEEN; INSERT: it is not there, *at is the
+// shared-memory address of the first empty entry and *bucket the bucket;
+// OVERFLOW: it is not there and cannot go there.  No branches with tags: a warp's lanes mostly
+// differ in the outcome, and each divergent branch costs more than computing all of it.
+enum { VISIT_SEEN = 0, VISIT_INSERT = 1, VISIT_OVERFLOW = 2 };
+
+__device__ __forceinline__ int probe_tags(const VisitTab &vt, uint32_t tab, int32_t e, uint32_t *at, uint32_t *bucket,
+                                          uint32_t *neu)
+{
+    const uint32_t y = (uint32_t)e * vt.mul;
+    const uint32_t b = y >> (32 - vt.bb);
+    const uint4 w = lds128(tab + (b << 4));
+    // 0 is never an entry: with 16-bit tags the ids of tag 0 always take the overflow
+    const uint32_t tg = ((y << vt.bb) >> (32 - vt.tb)) + (vt.tb < 16);
+    const uint32_t tt = __byte_perm(tg, 0, 0x1010);
+    const uint32_t has = (zero16(w.x ^ tt) | zero16(w.y ^ tt)) | (zero16(w.z ^ tt) | zero16(w.w ^ tt));
+    const uint32_t room = __popc((zero16(w.x) | (zero16(w.y) >> 1)) | ((zero16(w.z) >> 2) | (zero16(w.w) >> 3)));
+    *at = tab + (b << 4) + 16 - 2 * room;                // entries fill in order
+    *bucket = b;
+    *neu = tg;
+    const int r = room == 0 || tg == 0 ? VISIT_OVERFLOW : VISIT_INSERT;
+    return e < 0 || (has != 0 && tg != 0) ? VISIT_SEEN : r;
+}
+
+// With ids in the buckets, a full one continuing in the next; closed: nothing is inserted.
+__device__ __forceinline__ int probe_ids(const VisitTab &vt, uint32_t tab, int32_t e, bool closed, uint32_t *at,
+                                         uint32_t *bucket, uint32_t *neu)
+{
+    const uint32_t v = (uint32_t)e + 1;
+    uint32_t b = ((uint32_t)e * vt.mul) >> (32 - vt.bb);
+    *neu = v;
+    if (e < 0) return VISIT_SEEN;
+    for (;;) {                                           // ends: the table is at most three quarters full
+        const uint4 w = lds128(tab + b * 16);
+        if (w.x == v || w.y == v || w.z == v || w.w == v) return VISIT_SEEN;
+        if (w.w == 0) {
+            *at = tab + b * 16 + 4 * ((w.x != 0) + (w.y != 0) + (w.z != 0));
+            *bucket = b;
+            return closed ? VISIT_OVERFLOW : VISIT_INSERT;
+        }
+        b = (b + 1) & ((1u << vt.bb) - 1);
+    }
+}
+
+template <bool TAG>
+__device__ __forceinline__ int bucket_probe(const VisitTab &vt, uint32_t tab, int32_t e, bool closed, uint32_t *at,
+                                            uint32_t *bucket, uint32_t *neu)
+{
+    if (TAG) return probe_tags(vt, tab, e, at, bucket, neu);
+    return probe_ids(vt, tab, e, closed, at, bucket, neu);
+}
+template <bool TAG>
+__device__ __forceinline__ void bucket_store(uint32_t at, uint32_t v)
+{
+    if (TAG) asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"((unsigned short)v) : "memory");
+    else asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+
+// State of a query's visited set (warp-uniform).
+struct Visited {
+    unsigned char *tab;            // buckets
+    uint32_t tab_s, own_s;         // shared-memory addresses of the buckets and the owner bytes
+    int32_t *stash, *spill;        // overflow of the buckets: shared, then global
+    int hcount, scount;            // ids counted to the shared and to the global limit
+    int ocount;                    // ids in the stash
+    bool spilled, stash_full;      // counting to the global limit; overflow goes to spill
+
+    __device__ __forceinline__ void clear(const VisitTab &vt, int lane)
+    {
+#pragma unroll 1
+        for (uint32_t i = lane; i < vt.bytes / 16; i += 32) reinterpret_cast<uint4 *>(tab)[i] = make_uint4(0, 0, 0, 0);
+        if (vt.stash_log >= 0)
+#pragma unroll 1
+            for (int i = lane; i < (1 << vt.stash_log) / 4; i += 32)
+                reinterpret_cast<int4 *>(stash)[i] = make_int4(-1, -1, -1, -1);
+        hcount = scount = ocount = 0;
+        spilled = stash_full = false;
+    }
+    // the level-0 entry node (one lane, into the cleared set)
+    __device__ __forceinline__ void first(const VisitTab &vt, int32_t e, int lane)
+    {
+        hcount = 1;
+        if (lane == 0) {
+            uint32_t at = 0, b = 0, nw = 0;
+            const int r = vt.tag ? probe_tags(vt, tab_s, e, &at, &b, &nw) : probe_ids(vt, tab_s, e, false, &at, &b, &nw);
+            if (r != VISIT_INSERT) stash[hash32(e) & ((1 << vt.stash_log) - 1)] = e;
+            else if (vt.tag) bucket_store<true>(at, nw);
+            else bucket_store<false>(at, nw);
+        }
+        ocount = 1;                                      // (at most)
+    }
+};
+
+// Rare parts of the visited test, out of the way of the walk's code.  (Scalar arguments: a
+// reference would put the walk's state in memory.)
+static __device__ __noinline__ void clear_spill(int32_t *spill, int spill_log, int lane)
+{
+#pragma unroll 1
+    for (int i = lane; i < (1 << spill_log) / 4; i += 32)
+        reinterpret_cast<int4 *>(spill)[i] = make_int4(-1, -1, -1, -1);
+    __syncwarp();
+}
+// Id e into the overflow tables: the stash (stash_log >= 0) while it takes ids, else the global
+// table; true if it was in neither.
+static __device__ __noinline__ bool overflow_insert(int32_t e, int32_t *stash, int stash_log, bool stash_full, int32_t *spill,
+                                             int spill_log)
+{
+    if (stash_log >= 0) {
+        if (!stash_full) return table_insert(e, stash, stash_log, 0);
+        if (table_find(e, stash, stash_log, 0)) return false;
+    }
+    return table_insert(e, spill, spill_log, 3);
+}
+
+// Tests and inserts the adjacency rows of NR nodes (ev[u]: this lane's entry of row u, -1: none);
+// appends the ids seen for the first time to slot[ns...] and returns their number.  The caller
+// has checked the limits for all rows.  Insertion without atomics (one warp owns the table, and a
+// compare-and-swap on random shared addresses takes 180 cycles alone and 1,024 with 16 warps per
+// SM): in each round the lanes that want to insert write their code to their bucket's owner byte
+// (shared by buckets OWNERS apart), and the one that is read back stores its entry; the others look again, so an id in two rows
+// (or twice in one) is fresh once.  Two rounds are typical (four rows bring about 36 new ids,
+// some of them twice, to 256 buckets).
+template <bool TAG, int NR>
+__device__ __forceinline__ int visit_rows(Visited &V, const VisitTab &vt, int spill_log, const int32_t (&ev)[NR],
+                                          int32_t *slot, int ns, int lane)
+{
+    const bool closed = !TAG && V.spilled;
+    unsigned todo = 0, fresh = 0, over = 0;              // bit u: row u's entry
+#pragma unroll
+    for (int u = 0; u < NR; u++) todo |= (unsigned)(ev[u] >= 0) << u;
+    do {
+        uint32_t at[NR], own[NR] = {}, nw[NR];
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            const int r = bucket_probe<TAG>(vt, V.tab_s, (todo >> u) & 1 ? ev[u] : -1, closed, &at[u], &own[u], &nw[u]);
+            over |= (unsigned)(r == VISIT_OVERFLOW) << u;
+            if (r != VISIT_INSERT) todo &= ~(1u << u);
+            own[u] = V.own_s + (own[u] & (OWNERS - 1));
+        }
+#pragma unroll
+        for (int u = 0; u < NR; u++)
+            if ((todo >> u) & 1)
+                asm volatile("st.shared.u8 [%0], %1;" ::"r"(own[u]), "r"(lane | (u << 5)) : "memory");
+        __syncwarp();
+        unsigned won = 0;
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            uint32_t c = 0xff;
+            if ((todo >> u) & 1) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(c) : "r"(own[u]) : "memory");
+            won |= (unsigned)(c == (uint32_t)(lane | (u << 5))) << u;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < NR; u++)
+            if ((won >> u) & 1) bucket_store<TAG>(at[u], nw[u]);
+        fresh |= won;
+        todo &= ~won;
+        __syncwarp();
+    } while (__any_sync(FULL, todo != 0));
+    if (__any_sync(FULL, over != 0)) {
+#pragma unroll 1
+        for (int u = 0; u < NR; u++) {
+            const unsigned ov = __ballot_sync(FULL, (over >> u) & 1);
+            if (!ov) continue;
+            int32_t e = ev[0];
+#pragma unroll
+            for (int i = 1; i < NR; i++) e = u == i ? ev[i] : e;
+            if (TAG && !V.stash_full && V.ocount + __popc(ov) > shared_visited_cap(1 << vt.stash_log)) {
+                V.stash_full = true;
+                clear_spill(V.spill, spill_log, lane);
+            }
+            if ((over >> u) & 1)
+                fresh |= (unsigned)overflow_insert(e, V.stash, TAG ? vt.stash_log : -1, V.stash_full, V.spill, spill_log) << u;
+            if (!V.stash_full) V.ocount += __popc(ov);   // (at most)
+            __syncwarp();
+        }
+    }
+    const unsigned lt_mask = (1u << lane) - 1;
+    int n = ns;
+#pragma unroll
+    for (int u = 0; u < NR; u++) {
+        const bool f = (fresh >> u) & 1;
+        const unsigned m = __ballot_sync(FULL, f);
+        if (f) slot[n + __popc(m & lt_mask)] = ev[u];
+        n += __popc(m);
+    }
+    return n - ns;
+}
+
+// The rows of nodes sel[0..cnt) with ids in the buckets (very large indexes, table sizes asked for).
+static __device__ __noinline__ int visit_rows_ids(uint32_t tab, uint32_t owners, int bb, int32_t *spill, int spill_log,
+                                                  bool spilled, const int32_t *adj0, const int32_t *sel, int cnt,
+                                                  int32_t *slot, int ns, int lane)
+{
+    VisitTab vt{};
+    vt.bb = bb;
+    vt.mul = VISIT_MUL;
+    vt.stash_log = -1;
+    Visited V{};
+    V.tab_s = tab;
+    V.own_s = owners;
+    V.spill = spill;
+    V.spilled = spilled;
+    int32_t ev[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) ev[u] = u < cnt ? __ldg(adj0 + (int64_t)sel[u] * DEG + lane) : -1;
+    return visit_rows<false, 4>(V, vt, spill_log, ev, slot, ns, lane);
+}
+
+// Members of the sorted list W (wn keys) below k: four-way search, three reads a step in flight
+// together (a binary search would wait for twice as many dependent reads).
+__device__ __forceinline__ int members_below(const uint64_t *W, int wn, uint64_t k)
+{
+    int lo = 0;
+#pragma unroll 1
+    for (int s = 1 << ((31 - __clz(wn)) & ~1); s; s >>= 2) {
+        int c = 0;
+#pragma unroll
+        for (int j = 1; j < 4; j++) {
+            const int i = lo + j * s - 1;
+            if (i < wn) c += W[i] < k;
+        }
+        lo += c * s;
+    }
+    return lo;
+}
+
+// Merges the nc candidates of a step (keys cand[0..nc), distinct, in any order; room for three
+// more) into the sorted list W of wn keys in place, keeping the efp smallest; returns the new
+// length and in *first_new the lowest place a candidate took.  A candidate's place is the number
+// of candidates and of members below it (a count over the candidates, a search in W).  The
+// places not taken hold the members in order, so from the last 32 places down every place finds
+// its member from the number of candidates placed below it (one OR over the warp), and no member
+// searches; members only move up, so the places below are still the old ones.  Up to 32
+// candidates (nearly every step) stay in registers; else place[] keeps their places.
+__device__ __forceinline__ int merge_step(uint64_t *W, int wn, int efp, uint64_t *cand, int nc, int32_t *place, int lane,
+                                          int *first_new)
+{
+    const int wn2 = min(efp, wn + nc);
+    if (lane < 3) cand[nc + lane] = ~0ull;               // the count below takes four at a time
+    __syncwarp();
+    const bool one = nc <= 32;
+    int at = 0x7fffffff, lowest = 0x7fffffff;
+    uint64_t k = 0;
+#pragma unroll 1
+    for (int m0 = lane; m0 < nc; m0 += 32) {
+        k = cand[m0];
+        at = members_below(W, wn, k);
+#pragma unroll 1
+        for (int m = 0; m < nc; m += 4) {
+            const ulonglong2 c0 = *reinterpret_cast<const ulonglong2 *>(cand + m);
+            const ulonglong2 c1 = *reinterpret_cast<const ulonglong2 *>(cand + m + 2);
+            at += (c0.x < k) + (c0.y < k) + (c1.x < k) + (c1.y < k);
+        }
+        if (!one) place[m0] = at;
+        lowest = min(lowest, at);
+    }
+    lowest = (int)__reduce_min_sync(FULL, (unsigned)lowest);
+    *first_new = lowest;
+    int above = one ? __popc(__ballot_sync(FULL, at < wn2)) : 0;     // candidates placed before the end of the chunk
+    if (!one) {
+#pragma unroll 1
+        for (int m0 = 0; m0 < nc; m0 += 32) above += __popc(__ballot_sync(FULL, m0 + lane < nc && place[m0 + lane] < wn2));
+    }
+#pragma unroll 1
+    for (int c0 = (wn2 - 1) & ~31; c0 >= (lowest & ~31); c0 -= 32) {
+        unsigned mine = 0;
+        if (one) {
+            if (at >= c0 && at < min(c0 + 32, wn2)) mine = 1u << (at - c0);
+        } else {
+#pragma unroll 1
+            for (int m0 = lane; m0 < nc; m0 += 32) {
+                const int o = place[m0] - c0;
+                if (o >= 0 && o < min(32, wn2 - c0)) mine |= 1u << o;
+            }
+        }
+        const unsigned mask = __reduce_or_sync(FULL, mine);
+        const int t = c0 + lane, before = above - __popc(mask);
+        const bool member = !((mask >> lane) & 1) && t < wn2;
+        uint64_t key = 0;
+        if (member) key = W[t - before - __popc(mask & ((1u << lane) - 1))];
+        __syncwarp();
+        if (member) W[t] = key;
+        above = before;
+        __syncwarp();
+    }
+    if (one) {
+        if (at < wn2) W[at] = k;
+    } else {
+#pragma unroll 1
+        for (int m0 = lane; m0 < nc; m0 += 32)
+            if (place[m0] < wn2) W[place[m0]] = cand[m0];
+    }
+    return wn2;
+}
+
+// The codebooks of a walk or descent kernel into shared memory: the level-1 one and, for the full
+// walk in FP16, the level-2 one behind it (FP32: read through the cache, returned as *C2).
+template <int M1, int D1, typename CT, bool FQ, bool TAB>
+__device__ __forceinline__ void load_codebooks(const WalkArgs &a, unsigned char *smem, const CT **C2)
+{
+    *C2 = nullptr;
+    if constexpr (!TAB)
+        copy_async(smem, sizeof(CT) == 4 ? (const void *)a.C1 : (const void *)a.C1h, walk_c1_bytes(a.d, M1, D1, sizeof(CT)));
+    if constexpr (FQ && sizeof(CT) == 2) {
+        unsigned char *c2 = smem + walk_c1_bytes(a.d, M1, D1, sizeof(CT));
+        copy_async(c2, a.C2h, walk_c2_bytes(a.d, M1, D1));
+        *C2 = reinterpret_cast<const CT *>(c2);
+    } else if constexpr (FQ) {
+        *C2 = reinterpret_cast<const CT *>(a.C2);
+    }
+    copy_wait();
+    __syncthreads();
 }
 
 // TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
 // [256][M1] (FP16, built by table_kernel) in shared memory and scores nodes by table lookups.
 template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
-__global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArgs a)
+__global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = a.d;
     // the level-1 codebook, shared by every warp of the CTA
     CT *C1s = reinterpret_cast<CT *>(smem_raw);
-    if constexpr (!TAB) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(sizeof(CT) == 4 ? a.C1 : (const void *)a.C1h);
-        uint4 *dst = reinterpret_cast<uint4 *>(C1s);
-        const int n16 = (int)(walk_c1_bytes(d, M1, D1, sizeof(CT)) / 16);
-        for (int i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = __ldg(src + i);
-    }
-    // full walk: C2 in shared memory (FP16) or read through the cache (FP32)
-    const CT *C2 = nullptr;
-    if constexpr (FQ) {
-        if constexpr (sizeof(CT) == 2) {
-            CT *C2s = reinterpret_cast<CT *>(smem_raw + walk_c1_bytes(d, M1, D1, sizeof(CT)));
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.C2h);
-            for (int i = threadIdx.x; i < 256 * d * 2 / 16; i += blockDim.x) reinterpret_cast<uint4 *>(C2s)[i] = __ldg(src + i);
-            C2 = C2s;
-        } else {
-            C2 = reinterpret_cast<const CT *>(a.C2);
-        }
-    }
-    __syncthreads();
-    const WalkSmem L = walk_smem(M1, d, a.efcap, a.hash_log, a.beam, a.yq_in == nullptr, FQ ? a.M2P : 0);
+    const CT *C2;
+    load_codebooks<M1, D1, CT, FQ, TAB>(a, smem_raw, &C2);
+    const WalkSmem L = walk_smem(M1, d, a.efcap, a.vt, a.beam, a.yq_in == nullptr, FQ ? a.M2P : 0);
     constexpr size_t TABB = TAB ? (size_t)256 * M1 * 2 : 0;            // the query's table
     unsigned char *base = smem_raw + (TAB ? 0 : walk_cb_bytes(d, M1, D1, sizeof(CT), FQ)) + (size_t)warp * (L.total + TABB);
     if constexpr (TAB) C1s = reinterpret_cast<CT *>(base + L.total);
     float *yq = reinterpret_cast<float *>(base + L.yq);
     uint8_t *stage = base + L.stage;
-    uint64_t *wkey = reinterpret_cast<uint64_t *>(base + L.wkey);
-    uint8_t *wflag = base + L.wflag;
+    uint64_t *W = reinterpret_cast<uint64_t *>(base + L.wkey);
     uint64_t *cand = reinterpret_cast<uint64_t *>(base + L.cand);
-    uint64_t *cuns = reinterpret_cast<uint64_t *>(base + L.cunsorted);
+    int32_t *sel = reinterpret_cast<int32_t *>(base + L.sel);
     int32_t *slot = reinterpret_cast<int32_t *>(base + L.slot);
-    int32_t *rowbuf = reinterpret_cast<int32_t *>(base + L.rowbuf);
-    int32_t *hash = reinterpret_cast<int32_t *>(base + L.hash);
-    const int H = 1 << a.hash_log;
+    const int SR = stage_rows(M1 + (FQ ? a.M2P : 0), a.beam, a.vt.tag);
     const int64_t gwarp = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-    int32_t *spill = a.spill + (gwarp << a.spill_log);
+    Visited V;
+    V.tab = base + L.hash;
+    V.tab_s = (uint32_t)__cvta_generic_to_shared(V.tab);
+    V.stash = reinterpret_cast<int32_t *>(base + L.hash + a.vt.bytes);
+    V.own_s = (uint32_t)__cvta_generic_to_shared(base + L.stage);
+    const int H = 1 << a.hash_log;
+    const int my_slot = chunk_slot<M1>(lane);
     const unsigned lt_mask = (1u << lane) - 1;
 
     for (;;) {
@@ -588,6 +1045,7 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
         qi = __shfl_sync(FULL, qi, 0);
         if (qi >= a.nq) break;
         const int64_t q = a.order ? (int64_t)__ldg(a.order + qi) : qi;
+        V.spill = a.spill + ((a.spill_tables >= a.nq ? qi : gwarp) << a.spill_log);
         // this query's ef' = max(ef, k)
         const int efp = a.efq ? max(min(max(__ldg(a.efq + q), 1), a.efp), a.k) : a.efp;
         if constexpr (TAB) {
@@ -603,36 +1061,27 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
             // computed by rotate_kernel
         } else if (a.Q8) {
             const uint8_t *y = a.Q8 + q * d;
+#pragma unroll 1
             for (int t = lane; t < d; t += 32) {
                 float s = 0.f;
+#pragma unroll 4
                 for (int u = 0; u < d; u++) s = fmaf(__ldg(a.Rt + (int64_t)u * d + t), (float)__ldg(y + u), s);
                 yq[t] = s;
             }
         } else {
             const float *y = a.Q + q * d;
+#pragma unroll 1
             for (int t = lane; t < d; t += 32) {
                 float s = 0.f;
+#pragma unroll 4
                 for (int u = 0; u < d; u++) s = fmaf(__ldg(a.Rt + (int64_t)u * d + t), __ldg(y + u), s);
                 yq[t] = s;
             }
         }
-        if (a.mode != 1)
-            for (int i = lane; i < H; i += 32) hash[i] = -1;
+        V.clear(a.vt, lane);
         __syncwarp();
         LaneGeo<M1, D1> g;
-#pragma unroll
-        for (int k = 0; k < LaneGeo<M1, D1>::NSUB; k++) {
-            const int j = M1 == 16 ? (lane & 15) : lane + 32 * k;
-            g.j[k] = j;
-            g.off[k] = a.s1.off[j];
-            g.len[k] = a.s1.len[j];
-#pragma unroll
-            for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++) {
-                g.y[k][u] = u < g.len[k] ? yrot[g.off[k] + u] : 0.f;
-                g.m2[k][u] = FQ && u < g.len[k] ? a.sub2[g.off[k] + u] : 0;
-            }
-        }
-        int my_slot;
+        g.init(a.s1, yrot, FQ ? a.sub2 : nullptr, d, lane);
         // One loop runs the greedy descent of the upper levels (Section 2) and then the level-0
         // best-first search.  Each iteration gathers the nodes to score in slot[] and scores
         // them at a single call site, so the kernel holds one copy of the scoring code.
@@ -642,9 +1091,8 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
         int lvl = a.max_level;             // upper level being descended
         int phase = 0;                     // 0: entry point, 1: upper levels, 2: level 0
         int wn = 1;
-        bool spilled = false, failed = false;
-        int32_t hcount = 1, scount = 0;
-        int scan_from = 0;
+        bool failed = false;
+        int scan_from = 0;                 // every member of W before it is expanded
         const int B = a.beam;              // level-0 expansions per step; 1 = the plain walk
         if (a.mode == 2) {
             // level 0 from the entry node the descent launch recorded (as at its end below)
@@ -652,19 +1100,13 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
             dcur = __ldg(a.seed_d + q);
             n_up = __ldg(a.seed_up + q);
             phase = 2;
-            if (lane == 0) {
-                wkey[0] = make_key(dcur, cur);
-                wflag[0] = 0;
-                hash[hash32(cur) & (H - 1)] = cur;
-            }
+            if (lane == 0) W[0] = walk_key(dcur, cur);
+            V.first(a.vt, cur, lane);
             n_dist = 1;
             __syncwarp();
         }
         for (;;) {
-            uint64_t *W = wkey;
-            uint8_t *F = wflag;
-            int ns = 0, pos0 = 0;
-            uint64_t ckey0 = 0;
+            int ns = 0;
             if (phase == 0) {
                 if (lane == 0) slot[0] = cur;
                 ns = 1;
@@ -677,155 +1119,88 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
                 n_up += ns;
             } else {
                 if (a.tcap > 0 && n_dist >= a.tcap) break;     // search-time cap T (Section 3.1)
-                // the B best unexpanded members of W: lane i < nb holds the i-th one's position
-                int nb = 0, my_pos = -1;
+                // the B best unexpanded members of W, marked expanded, their ids in sel[]
+                int nb = 0;
+#pragma unroll 1
                 for (int b0 = scan_from; b0 < wn && nb < B; b0 += 32) {
                     const int p = b0 + lane;
-                    unsigned m = __ballot_sync(FULL, p < wn && !F[p]);
-                    while (m && nb < B) {
-                        if (lane == nb) my_pos = b0 + __ffs(m) - 1;
-                        nb++;
-                        m &= m - 1;
+                    const uint64_t key = p < wn ? W[p] : 1;
+                    const bool open = !(key & 1);
+                    const unsigned m = __ballot_sync(FULL, open);
+                    const int i = nb + __popc(m & lt_mask);
+                    if (open && i < B) {
+                        sel[i] = walk_id(key);
+                        W[p] = key | 1;
                     }
+                    if (nb == 0 && m) scan_from = b0;
+                    nb += __popc(m);
                 }
+                nb = min(nb, B);
                 if (nb == 0) break;
-                pos0 = __shfl_sync(FULL, my_pos, 0);
-                ckey0 = W[pos0];
-                const int32_t my_c = lane < nb ? key_id(W[my_pos]) : -1;
-                __syncwarp();
-                if (lane < nb) F[my_pos] = 1;
                 n_expand += nb;
-                // their adjacency rows, all loads in flight together
-                for (int r = 0; r < nb; r++) {
-                    const int32_t cr = __shfl_sync(FULL, my_c, r);
-                    rowbuf[r * DEG + lane] = a.adj0[(int64_t)cr * DEG + lane];
-                }
                 __syncwarp();
-                // visited test row by row (row order, then slot order); fresh nodes are appended
-                if (!spilled && hcount + 32 * nb <= shared_visited_cap(H)) {
-                    // every row fits in the shared table without a switch to the spill table: the
-                    // first probes of up to 4 rows are issued together, then each row is resolved
-                    // in row order (a node in two rows probes the same bucket first, so it is
-                    // fresh in the earlier row)
-                    const uint32_t Hm = (uint32_t)H - 1;
-                    for (int r0 = 0; r0 < nb; r0 += 4) {
-                        int32_t ev[4], ov[4];
-#pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            ev[u] = r0 + u < nb ? rowbuf[(r0 + u) * DEG + lane] : -1;
-                            ov[u] = ev[u] >= 0 ? atomicCAS(hash + (hash32(ev[u]) & Hm), -1, ev[u]) : 0;
+                if (nb > 4 && lane >= 4 && lane < nb)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(a.adj0 + (int64_t)sel[lane] * DEG));
+                // their adjacency rows through the visited test, four rows at a time while the
+                // limits leave room for all of them, else row by row; fresh nodes are appended
+                const int half = (1 << a.spill_log) / 2;
+#pragma unroll 1
+                for (int r0 = 0; r0 < nb;) {
+                    int cnt = min(4, nb - r0);
+                    if (V.spilled ? V.scount + 32 * cnt > half : V.hcount + 32 * cnt > shared_visited_cap(H)) {
+                        cnt = 1;
+                        if (!V.spilled && V.hcount + 32 > shared_visited_cap(H)) {
+                            V.spilled = true;            // from here on counted to the global limit
+                            if (!a.vt.tag) clear_spill(V.spill, a.spill_log, lane);
                         }
-#pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            if (r0 + u >= nb) break;
-                            const int32_t e = ev[u];
-                            bool fresh = e >= 0 && ov[u] == -1;
-                            if (e >= 0 && ov[u] != -1 && ov[u] != e) {
-                                // collision: continue the probe sequence
-                                uint32_t h = hash32(e) & Hm;
-                                for (uint32_t p = 1; p <= Hm; p++) {
-                                    h = (h + p) & Hm;
-                                    const int32_t old = atomicCAS(hash + h, -1, e);
-                                    if (old == -1) { fresh = true; break; }
-                                    if (old == e) break;
-                                }
-                            }
-                            const unsigned fm = __ballot_sync(FULL, fresh);
-                            if (fresh) slot[ns + __popc(fm & lt_mask)] = e;
-                            const int nf = __popc(fm);
-                            ns += nf;
-                            n_dist += nf;
-                            hcount += nf;
+                        if (V.spilled && V.scount + 32 > half) {
+                            failed = true;
+                            break;
                         }
                     }
-                } else if (spilled && scount + 32 * nb <= (1 << a.spill_log) / 2) {
-                    // spilled, and every row fits in the global table: the shared table is only
-                    // read; the first global probes of up to 4 rows are issued together, then
-                    // each row is resolved in row order (as above)
-                    const uint32_t Hm = (uint32_t)H - 1, Sm = (1u << a.spill_log) - 1;
-                    for (int r0 = 0; r0 < nb; r0 += 4) {
-                        int32_t ev[4], ov[4];
-                        bool seen[4];
+                    int nf;
+                    if (!a.vt.tag) {
+                        nf = visit_rows_ids(V.tab_s, V.own_s, a.vt.bb, V.spill, a.spill_log, V.spilled, a.adj0, sel + r0,
+                                            cnt, slot, ns, lane);
+                    } else if (cnt == 1) {
+                        const int32_t ev[1] = {__ldg(a.adj0 + (int64_t)sel[r0] * DEG + lane)};
+                        nf = visit_rows<true, 1>(V, a.vt, a.spill_log, ev, slot, ns, lane);
+                    } else {
+                        int32_t ev[4];
 #pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            ev[u] = r0 + u < nb ? rowbuf[(r0 + u) * DEG + lane] : -1;
-                            seen[u] = false;
-                            if (ev[u] >= 0) {
-                                uint32_t h = hash32(ev[u]) & Hm;
-                                for (uint32_t p = 0; p <= Hm; p++) {
-                                    const int32_t v = hash[h];
-                                    if (v == ev[u]) { seen[u] = true; break; }
-                                    if (v == -1) break;
-                                    h = (h + p + 1) & Hm;
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; u++)
-                            ov[u] = ev[u] >= 0 && !seen[u] ? atomicCAS(spill + ((hash32(ev[u]) >> 3) & Sm), -1, ev[u]) : 0;
-#pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            if (r0 + u >= nb) break;
-                            const int32_t e = ev[u];
-                            bool fresh = e >= 0 && !seen[u] && ov[u] == -1;
-                            if (e >= 0 && !seen[u] && ov[u] != -1 && ov[u] != e) {
-                                uint32_t h = (hash32(e) >> 3) & Sm;
-                                for (uint32_t p = 1; p <= Sm; p++) {
-                                    h = (h + p) & Sm;
-                                    const int32_t old = atomicCAS(spill + h, -1, e);
-                                    if (old == -1) { fresh = true; break; }
-                                    if (old == e) break;
-                                }
-                            }
-                            const unsigned fm = __ballot_sync(FULL, fresh);
-                            if (fresh) slot[ns + __popc(fm & lt_mask)] = e;
-                            const int nf = __popc(fm);
-                            ns += nf;
-                            n_dist += nf;
-                            scount += nf;
-                        }
+                        for (int u = 0; u < 4; u++) ev[u] = u < cnt ? __ldg(a.adj0 + (int64_t)sel[r0 + u] * DEG + lane) : -1;
+                        nf = visit_rows<true, 4>(V, a.vt, a.spill_log, ev, slot, ns, lane);
                     }
-                } else for (int r = 0; r < nb; r++) {
-                    // switch to the global table before the shared one passes its limit
-                    if (!spilled && hcount + 32 > shared_visited_cap(H)) {
-                        spilled = true;
-                        for (int i = lane; i < (1 << a.spill_log); i += 32) spill[i] = -1;
-                        __syncwarp();
-                    }
-                    if (spilled && scount + 32 > (1 << a.spill_log) / 2) {
-                        failed = true;
-                        break;
-                    }
-                    const int32_t e = rowbuf[r * DEG + lane];
-                    const bool fresh = e >= 0 && visit(e, hash, a.hash_log, spilled, spill, a.spill_log);
-                    const unsigned fm = __ballot_sync(FULL, fresh);
-                    if (fresh) slot[ns + __popc(fm & lt_mask)] = e;
-                    const int nf = __popc(fm);
                     ns += nf;
                     n_dist += nf;
-                    if (spilled) scount += nf; else hcount += nf;
+                    if (V.spilled) V.scount += nf; else V.hcount += nf;
+                    r0 += cnt;
                 }
                 if (failed) break;
-                __syncwarp();
-                if (ns == 0) { scan_from = pos0; continue; }
+                if (ns == 0) {
+                    __syncwarp();
+                    continue;
+                }
             }
-            __syncwarp();
             // score the gathered nodes 32 at a time: the upper levels keep the best, level 0
-            // keeps those that can enter W
-            const uint64_t wmax = (phase == 2 && wn == efp) ? W[wn - 1] : ~0ull;
-            uint64_t best = ~0ull;
+            // collects those that can enter W and merges them into it
+            uint32_t bd = ~0u, bi = ~0u;
+            const uint64_t wmax = phase == 2 && wn == efp ? W[wn - 1] : ~0ull;
             int nc = 0;
+#pragma unroll 1
             for (int ch = 0; ch < ns; ch += 32) {
+                const int at = ch % SR;                  // place in the staging area
+                if (at == 0) stage_codes<M1, FQ>(stage, SR, a.codes1, a.codes2b, a.M2P, slot + ch, min(SR, ns - ch), lane);
                 const int nf = min(32, ns - ch);
-                const float de = score_nodes<M1, D1, CT, FQ, TAB>(C1s, stage, a.codes1, slot + ch, nf, d, g, lane, &my_slot,
-                                                             C2, a.codes2b, a.M2P);
-                uint64_t k = my_slot < nf ? make_key(de, slot[ch + my_slot]) : ~0ull;
-                if (phase < 2) {
-                    best = warp_min64(k);                   // at most 32 nodes here
+                const float de = score_staged<M1, D1, CT, FQ, TAB>(C1s, stage + at * M1, stage + SR * M1 + at * a.M2P, nf, d, g,
+                                                                   lane, C2, a.M2P);
+                const int32_t id = my_slot < nf ? slot[ch + my_slot] : -1;
+                if (phase < 2) {                         // at most 32 nodes here
+                    warp_best(id >= 0 ? __float_as_uint(de) : ~0u, (uint32_t)id, &bd, &bi);
                 } else {
-                    if (k >= wmax) k = ~0ull;
-                    const unsigned km = __ballot_sync(FULL, k != ~0ull);
-                    if (k != ~0ull) cuns[nc + __popc(km & lt_mask)] = k;
+                    const uint64_t k = id >= 0 ? walk_key(de, id) : ~0ull;
+                    const unsigned km = __ballot_sync(FULL, k < wmax);
+                    if (k < wmax) cand[nc + __popc(km & lt_mask)] = k;
                     nc += __popc(km);
                 }
             }
@@ -833,118 +1208,48 @@ __global__ void __launch_bounds__(MAX_WALK_WARPS * 32) walk_kernel(const WalkArg
             if (phase < 2) {
                 bool enter0 = false;
                 if (phase == 0) {
-                    dcur = key_dist(best);
+                    dcur = __uint_as_float(bd);
                     if (lvl >= 1) {
                         n_up = 1;                           // the entry point's evaluation
                         phase = 1;
                     } else {
                         enter0 = true;
                     }
-                } else if (ns > 0 && best < make_key(dcur, cur)) {
-                    cur = key_id(best);                     // greedy move at this level
-                    dcur = key_dist(best);
+                } else if (ns > 0 && (bd < __float_as_uint(dcur) || (bd == __float_as_uint(dcur) && (int32_t)bi < cur))) {
+                    cur = (int32_t)bi;                      // greedy move at this level
+                    dcur = __uint_as_float(bd);
                 } else if (--lvl == 0) {
                     enter0 = true;
                 }
-                if (enter0 && a.mode == 1) {
-                    // descent only: record the level-0 entry for the second launch
-                    if (lane == 0) {
-                        a.seed[q] = cur;
-                        a.seed_d[q] = dcur;
-                        a.seed_up[q] = n_up;
-                    }
-                    break;
-                }
                 if (enter0) {
-                    // level 0: best-first search with result list W (sorted keys + expanded flags)
+                    // level 0: best-first search with the result list W (sorted keys)
                     phase = 2;
-                    if (lane == 0) {
-                        wkey[0] = make_key(dcur, cur);
-                        wflag[0] = 0;
-                        hash[hash32(cur) & (H - 1)] = cur;
-                    }
+                    if (lane == 0) W[0] = walk_key(dcur, cur);
+                    V.first(a.vt, cur, lane);
                     n_dist = 1;
                     __syncwarp();
                 }
-                continue;
-            }
-            if (nc == 0) { scan_from = pos0; continue; }
-            // order the candidates by rank (keys are distinct)
-            for (int m0 = lane; m0 < nc; m0 += 32) {
-                const uint64_t mk = cuns[m0];
-                int r = 0;
-                for (int m = 0; m < nc; m++) r += cuns[m] < mk;
-                cand[r] = mk;
-            }
-            __syncwarp();
-            // merge the nc candidates into W (wn keys) in place, keep ef': a candidate's place
-            // is its rank plus the members below it, a member's its index plus the candidates
-            // below it.  The candidates' places are taken first (into slot[], free after
-            // scoring); members only move up, so chunks of 32 move from the last one down,
-            // each read whole before it is written; the candidates are written last.
-            const int wn2 = min(efp, wn + nc);
-            int first_new = efp;
-            for (int m0 = lane; m0 < nc; m0 += 32) {
-                const uint64_t ck = cand[m0];
-                int lo = 0, hi = wn;                     // W members below the candidate
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (W[mid] < ck) lo = mid + 1; else hi = mid;
-                }
-                slot[m0] = m0 + lo;
-                if (m0 == 0) first_new = m0 + lo;
-            }
-            first_new = __shfl_sync(FULL, first_new, 0);
-            __syncwarp();
-            // members before the first candidate's place keep theirs
-            for (int c0 = (wn - 1) & ~31; c0 >= (first_new & ~31); c0 -= 32) {
-                const int p = c0 + lane;
-                uint64_t key = 0;
-                uint8_t f = 0;
-                int np = p;
-                if (p < wn) {
-                    key = W[p];
-                    f = F[p];
-                    int lo = 0, hi = nc;                 // candidates below key
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (cand[mid] < key) lo = mid + 1; else hi = mid;
-                    }
-                    np = p + lo;
-                }
-                __syncwarp();
-                if (np != p && np < wn2) { W[np] = key; F[np] = f; }
+            } else if (nc > 0) {
+                int first_new;
+                wn = merge_step(W, wn, efp, cand, nc, slot, lane, &first_new);
+                scan_from = min(scan_from, first_new & ~31);
                 __syncwarp();
             }
-            for (int m0 = lane; m0 < nc; m0 += 32) {
-                const int np = slot[m0];
-                if (np < wn2) { W[np] = cand[m0]; F[np] = 0; }
-            }
-            // everything before min(first new candidate, first expanded node's new place) is
-            // expanded
-            int below = 0;
-            for (int m = 0; m < nc; m++) below += cand[m] < ckey0;
-            scan_from = min(first_new, pos0 + below);
-            scan_from -= scan_from % 32;
-            wn = wn2;
-            __syncwarp();
         }
 
-        if (a.mode == 1) {
-            __syncwarp();
-            continue;
-        }
         // outputs
-        const uint64_t *W = wkey;
         if (a.refine) {
             if (!a.yq_in)
+#pragma unroll 1
                 for (int t = lane; t < d; t += 32) a.yq_out[q * d + t] = yq[t];
+#pragma unroll 1
             for (int i = lane; i < a.R; i += 32)
-                a.short_out[q * a.R + i] = (!failed && i < wn) ? key_id(W[i]) : -1;
+                a.short_out[q * a.R + i] = (!failed && i < wn) ? walk_id(W[i]) : -1;
         } else {
+#pragma unroll 1
             for (int i = lane; i < a.R; i += 32) {
                 bool ok = !failed && i < wn;
-                a.ids_out[q * a.R + i] = ok ? key_id(W[i]) : -1;
+                a.ids_out[q * a.R + i] = ok ? walk_id(W[i]) : -1;
                 a.dists_out[q * a.R + i] = ok ? key_dist(W[i]) : __int_as_float(0x7f800000);
             }
         }
@@ -986,29 +1291,14 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = a.d;
     CT *C1s = reinterpret_cast<CT *>(smem_raw);
-    if constexpr (!TAB) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(sizeof(CT) == 4 ? a.C1 : (const void *)a.C1h);
-        uint4 *dst = reinterpret_cast<uint4 *>(C1s);
-        const int n16 = (int)(walk_c1_bytes(d, M1, D1, sizeof(CT)) / 16);
-        for (int i = threadIdx.x; i < n16; i += blockDim.x) dst[i] = __ldg(src + i);
-    }
-    const CT *C2 = nullptr;
-    if constexpr (FQ) {
-        if constexpr (sizeof(CT) == 2) {
-            CT *C2s = reinterpret_cast<CT *>(smem_raw + walk_c1_bytes(d, M1, D1, sizeof(CT)));
-            const uint4 *src = reinterpret_cast<const uint4 *>(a.C2h);
-            for (int i = threadIdx.x; i < 256 * d * 2 / 16; i += blockDim.x) reinterpret_cast<uint4 *>(C2s)[i] = __ldg(src + i);
-            C2 = C2s;
-        } else {
-            C2 = reinterpret_cast<const CT *>(a.C2);
-        }
-    }
-    __syncthreads();
+    const CT *C2;
+    load_codebooks<M1, D1, CT, FQ, TAB>(a, smem_raw, &C2);
     const int m2p = FQ ? a.M2P : 0;
     unsigned char *base = smem_raw + (TAB ? 0 : walk_cb_bytes(d, M1, D1, sizeof(CT), FQ)) +
                           (size_t)warp * descent_smem_per_warp(M1, m2p);
     uint8_t *stage = base;
     int32_t *slot = reinterpret_cast<int32_t *>(base + align_up((size_t)32 * (M1 + m2p), 16));
+    const int my_slot = chunk_slot<M1>(lane);
     const unsigned lt_mask = (1u << lane) - 1;
 
     for (;;) {
@@ -1021,18 +1311,7 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
         // TAB: the query's ADC table [256][M1], read through L1 (a descent scores few nodes)
         const CT *T1 = TAB ? reinterpret_cast<const CT *>(a.tab + q * 256 * M1) : C1s;
         LaneGeo<M1, D1> g;
-#pragma unroll
-        for (int k = 0; k < LaneGeo<M1, D1>::NSUB; k++) {
-            const int j = M1 == 16 ? (lane & 15) : lane + 32 * k;
-            g.j[k] = j;
-            g.off[k] = a.s1.off[j];
-            g.len[k] = a.s1.len[j];
-#pragma unroll
-            for (int u = 0; u < LaneGeo<M1, D1>::DMAX; u++) {
-                g.y[k][u] = u < g.len[k] ? yrot[g.off[k] + u] : 0.f;
-                g.m2[k][u] = FQ && u < g.len[k] ? a.sub2[g.off[k] + u] : 0;
-            }
-        }
+        g.init(a.s1, yrot, FQ ? a.sub2 : nullptr, d, lane);
         // the entry point's evaluation, then steepest moves level by level (as walk_kernel)
         int32_t cur = a.ep, n_up = 0;
         float dcur = 0.f;
@@ -1050,24 +1329,22 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
                 if (e >= 0) slot[__popc(vm & lt_mask)] = e;
                 n_up += ns;
             }
-            __syncwarp();
-            uint64_t best = ~0ull;
+            uint32_t bd = ~0u, bi = ~0u;
             if (ns > 0) {
-                int my_slot;
-                const float de = score_nodes<M1, D1, CT, FQ, TAB>(T1, stage, a.codes1, slot, ns, d, g, lane, &my_slot,
-                                                                  C2, a.codes2b, a.M2P);
-                const uint64_t k = my_slot < ns ? make_key(de, slot[my_slot]) : ~0ull;
-                best = warp_min64(k);
+                stage_codes<M1, FQ>(stage, 32, a.codes1, a.codes2b, a.M2P, slot, ns, lane);
+                const float de = score_staged<M1, D1, CT, FQ, TAB>(T1, stage, stage + 32 * M1, ns, d, g, lane, C2, a.M2P);
+                const int32_t id = my_slot < ns ? slot[my_slot] : -1;
+                warp_best(id >= 0 ? __float_as_uint(de) : ~0u, (uint32_t)id, &bd, &bi);
             }
             __syncwarp();
             if (first) {
                 first = false;
-                dcur = key_dist(best);
+                dcur = __uint_as_float(bd);
                 if (lvl < 1) break;
                 n_up = 1;                                   // the entry point's evaluation
-            } else if (ns > 0 && best < make_key(dcur, cur)) {
-                cur = key_id(best);                         // greedy move at this level
-                dcur = key_dist(best);
+            } else if (ns > 0 && (bd < __float_as_uint(dcur) || (bd == __float_as_uint(dcur) && (int32_t)bi < cur))) {
+                cur = (int32_t)bi;                          // greedy move at this level
+                dcur = __uint_as_float(bd);
             } else if (--lvl == 0) {
                 break;
             }
@@ -1091,6 +1368,7 @@ static cudaError_t launch_descent(const WalkArgs &wa, int sms, int *wpc_out, int
     const size_t per = descent_smem_per_warp(M1, FQ ? wa.M2P : 0);
     if (c1 + per > MAX_SMEM_PER_BLOCK) return cudaErrorInvalidConfiguration;
     int wpc = (int)std::min<size_t>(MAX_DESCENT_WARPS, (MAX_SMEM_PER_BLOCK - c1) / per);
+    wpc = (int)std::min<int64_t>(wpc, std::max<int64_t>(1, (wa.nq + sms - 1) / sms));
     cudaError_t e = cudaFuncSetAttribute(descent_kernel<M1, D1, CT, FQ, TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)MAX_SMEM_PER_BLOCK);
     if (e != cudaSuccess) return e;
@@ -1133,8 +1411,10 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
 {
     size_t c1 = TAB ? 0 : walk_cb_bytes(wa.d, M1, D1, sizeof(CT), FQ);
     if (c1 + smem_per_warp > MAX_SMEM_PER_BLOCK) return cudaErrorInvalidConfiguration;
-    int wpc = (int)std::min<size_t>(MAX_WALK_WARPS, (MAX_SMEM_PER_BLOCK - c1) / smem_per_warp);
+    int wpc = (int)std::min<size_t>(walk_threads(D1, FQ) / 32, (MAX_SMEM_PER_BLOCK - c1) / smem_per_warp);
     if (want > 0) wpc = std::min(wpc, want);
+    // a batch that does not fill the GPU spreads over all SMs
+    wpc = (int)std::min<int64_t>(wpc, std::max<int64_t>(1, (wa.nq + num_sms - 1) / num_sms));
     size_t smem = c1 + smem_per_warp * wpc;
     // the attribute is an upper bound: set to the maximum, so plans made in any order (the
     // server plans at submission and launches later) all remain launchable
