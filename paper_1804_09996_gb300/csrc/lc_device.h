@@ -114,9 +114,7 @@ struct SearchPlan {
     bool full = false;                   // the walk scores the full two-level decode
     int wpc = 0, grid = 0;               // walk: warps per CTA, CTAs
     size_t per_warp = 0, smem = 0;
-    int rw = 0, rgrid = 0;               // refine: warps per CTA, CTAs
-    int qgrid = 0;                       // rotation: CTAs
-    size_t qsm = 0;                      // rotation: shared memory
+    int rw = 0, rgrid = 0, rteam = 1;    // refine: warps per CTA, CTAs, warps per query
     size_t rsm = 0;
     bool rboth = false;                  // both codebooks in shared memory
     bool ordered = false;                // two walk launches, level 0 in decreasing entry distance

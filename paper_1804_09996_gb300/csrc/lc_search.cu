@@ -25,6 +25,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "lc_walk.cuh"
 
@@ -55,6 +56,7 @@ struct RefineArgs {
     const float *yq;
     const int32_t *shortlist;
     int64_t nq;
+    int T;                          // warps per query
     int R, k, d, M1, M2P;           // M2P: padded row of the residual codes (codeword ids last)
     int BM, BK;                     // regression blocks, codewords per block (B: [BM][BK][9])
     const float *C1, *C2, *B;
@@ -70,64 +72,117 @@ struct RefineArgs {
 // Query rotation y' = R y (Section 3.3 / 5.1: OPQ rotates vectors and queries alike) for a
 // whole batch ahead of the walk.  Every output coordinate is the fixed-order sum over
 // u = 0..d-1 of R[t][u] y[u] (fmaf chain), the arithmetic of the walk's own rotation, so the
-// walk gives bit-identical results either way.  R^T sits in shared memory when it fits
-// (d <= 200); uint8 queries convert exactly to FP32.
-constexpr int ROT_Q = 16;           // queries per block step (independent FMA chains per thread)
-constexpr int ROT_THREADS = 128;
-__host__ __device__ inline bool rotate_rt_shared(int d) { return (size_t)d * d * 4 <= 160 * 1024; }
-__host__ __device__ inline size_t rotate_smem(int d)
+// walk gives bit-identical results whichever kernel rotates.  uint8 queries convert exactly to
+// FP32.  Both kernels also reset the search's query counter and status word, which saves two
+// launches.
+__device__ __forceinline__ float query_at(const float *Q, const uint8_t *Q8, int64_t i)
 {
-    return ((rotate_rt_shared(d) ? (size_t)d * d : 0) + (size_t)ROT_Q * d) * 4;
+    return Q8 ? (float)__ldg(Q8 + i) : __ldg(Q + i);
 }
 
-// A thread owns output coordinate t of ROT_Q queries at a time: ROT_Q independent chains,
-// with the queries' values read four at a time from ys [d][ROT_Q] (broadcast).
-__global__ void __launch_bounds__(ROT_THREADS) rotate_kernel(const float *Q, const uint8_t *Q8, int64_t nq, int d,
-                                                             const float *Rt, float *yq)
+// Small batches (and any d): a block takes QB queries, a thread owns output coordinates t of
+// all of them; R^T is read from L2, eight rows in flight.  Bound by that latency, and not by a
+// copy of R^T into shared memory first: 16 queries 18 -> 9 us.
+template <int QB>
+__global__ void __launch_bounds__(128) rotate_few_kernel(const float *Q, const uint8_t *Q8, int64_t nq, int d, const float *Rt,
+                                                         float *yq, unsigned long long *counter, int32_t *status)
+{
+    __shared__ __align__(16) float ys[256 * QB];         // [d][QB]
+    const int64_t q0 = (int64_t)blockIdx.x * QB;
+    if (blockIdx.x == 0 && threadIdx.x == 0) { *counter = 0; *status = 0; }
+    for (int i = threadIdx.x; i < QB * d; i += blockDim.x) {
+        const int qq = i / d, u = i - qq * d;
+        ys[u * QB + qq] = q0 + qq < nq ? query_at(Q, Q8, (q0 + qq) * d + u) : 0.f;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < d; t += blockDim.x) {
+        float acc[QB];
+#pragma unroll
+        for (int qq = 0; qq < QB; qq++) acc[qq] = 0.f;
+        int u = 0;
+        for (; u + 8 <= d; u += 8) {
+            float r[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) r[i] = __ldg(Rt + (int64_t)(u + i) * d + t);
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+#pragma unroll
+                for (int qq = 0; qq < QB; qq++) acc[qq] = fmaf(r[i], ys[(u + i) * QB + qq], acc[qq]);
+        }
+        for (; u < d; u++) {
+            const float r = __ldg(Rt + (int64_t)u * d + t);
+#pragma unroll
+            for (int qq = 0; qq < QB; qq++) acc[qq] = fmaf(r, ys[u * QB + qq], acc[qq]);
+        }
+#pragma unroll
+        for (int qq = 0; qq < QB; qq++)
+            if (q0 + qq < nq) yq[(q0 + qq) * d + t] = acc[qq];
+    }
+}
+
+// Large batches, d a multiple of 4 up to 200: a block takes ROT_Q queries; R^T and the queries
+// (transposed) sit in shared memory, and a thread owns 4 coordinates of 8 queries, so that three
+// 16-byte shared reads feed 32 multiply-adds (packed two at a time, the scalar roundings).
+// 100,000 queries of d = 96: 130 us with one coordinate of 16 queries per thread, 77 us now.
+constexpr int ROT_Q = 64;
+constexpr int ROT_S = ROT_Q + 4;    // row stride of the transposed queries (16-byte rows, fewer bank conflicts)
+constexpr int ROT_MIN = 4096;       // from here on: about half of the SMs have a block of ROT_Q queries
+__host__ __device__ inline bool rotate_tiled(int64_t nq, int d) { return d % 4 == 0 && d <= 200 && nq >= ROT_MIN; }
+__host__ __device__ inline size_t rotate_smem(int d) { return ((size_t)d * d + (size_t)ROT_S * d) * 4; }
+
+__global__ void __launch_bounds__(400) rotate_kernel(const float *Q, const uint8_t *Q8, int64_t nq, int d, const float *Rt,
+                                                     float *yq, unsigned long long *counter, int32_t *status)
 {
     extern __shared__ __align__(128) float rsm[];
-    const bool shared_rt = rotate_rt_shared(d);
-    float *ys = rsm + (shared_rt ? d * d : 0);
-    const float *R = Rt;
-    if (shared_rt) {
-        // 16-byte loads, several in flight per thread (R^T is cudaMalloc-aligned)
-        const int n4 = d * d / 4;
-#pragma unroll 6
-        for (int i = threadIdx.x; i < n4; i += blockDim.x)
-            reinterpret_cast<float4 *>(rsm)[i] = __ldg(reinterpret_cast<const float4 *>(Rt) + i);
-        for (int i = 4 * n4 + threadIdx.x; i < d * d; i += blockDim.x) rsm[i] = __ldg(Rt + i);
-        R = rsm;
+    float *ys = rsm + d * d;                             // [d][ROT_S]
+    if (blockIdx.x == 0 && threadIdx.x == 0) { *counter = 0; *status = 0; }
+    copy_async(rsm, Rt, (size_t)d * d * 4);              // (d * d a multiple of 4; cudaMalloc-aligned)
+    const int64_t q0 = (int64_t)blockIdx.x * ROT_Q;
+#pragma unroll 16
+    for (int i = threadIdx.x; i < ROT_Q * d; i += blockDim.x) {
+        const int qq = i / d, u = i - qq * d;
+        ys[u * ROT_S + qq] = q0 + qq < nq ? query_at(Q, Q8, q0 * d + i) : 0.f;
     }
-    for (int64_t q0 = (int64_t)blockIdx.x * ROT_Q; q0 < nq; q0 += (int64_t)gridDim.x * ROT_Q) {
-        const int nb = nq - q0 < ROT_Q ? (int)(nq - q0) : ROT_Q;
-        __syncthreads();                               // Rt loaded / previous step's ys consumed
+    copy_wait();
+    __syncthreads();
+    const int nt = d / 4, t0 = 4 * (threadIdx.x % nt), b0 = 8 * (threadIdx.x / nt);
+    unsigned long long acc[4][4] = {};                   // [query pair][coordinate]
 #pragma unroll 4
-        for (int i = threadIdx.x; i < ROT_Q * d; i += blockDim.x) {
-            const int qq = i / d, u = i - qq * d;
-            ys[u * ROT_Q + qq] = qq >= nb ? 0.f : Q8 ? (float)__ldg(Q8 + (q0 + qq) * d + u) : __ldg(Q + (q0 + qq) * d + u);
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < d; t += blockDim.x) {
-            float acc[ROT_Q];
+    for (int u = 0; u < d; u++) {
+        const float4 r = *reinterpret_cast<const float4 *>(rsm + u * d + t0);
+        const ulonglong2 ya = *reinterpret_cast<const ulonglong2 *>(ys + u * ROT_S + b0);
+        const ulonglong2 yb = *reinterpret_cast<const ulonglong2 *>(ys + u * ROT_S + b0 + 4);
+        const unsigned long long y[4] = {ya.x, ya.y, yb.x, yb.y};
+        const unsigned long long rr[4] = {pack2(r.x, r.x), pack2(r.y, r.y), pack2(r.z, r.z), pack2(r.w, r.w)};
 #pragma unroll
-            for (int qq = 0; qq < ROT_Q; qq++) acc[qq] = 0.f;
-#pragma unroll 4
-            for (int u = 0; u < d; u++) {
-                const float r = R[u * d + t];
-                const float4 *y4 = reinterpret_cast<const float4 *>(ys + u * ROT_Q);
+        for (int p = 0; p < 4; p++)
 #pragma unroll
-                for (int v = 0; v < ROT_Q / 4; v++) {
-                    const float4 y = y4[v];
-                    acc[4 * v + 0] = fmaf(r, y.x, acc[4 * v + 0]);
-                    acc[4 * v + 1] = fmaf(r, y.y, acc[4 * v + 1]);
-                    acc[4 * v + 2] = fmaf(r, y.z, acc[4 * v + 2]);
-                    acc[4 * v + 3] = fmaf(r, y.w, acc[4 * v + 3]);
-                }
-            }
+            for (int t = 0; t < 4; t++) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[p][t]) : "l"(rr[t]), "l"(y[p]));
+    }
 #pragma unroll
-            for (int qq = 0; qq < ROT_Q; qq++)
-                if (qq < nb) yq[(q0 + qq) * d + t] = acc[qq];
-        }
+    for (int p = 0; p < 4; p++) {
+        float4 a, b;
+        unpack2(acc[p][0], a.x, b.x);
+        unpack2(acc[p][1], a.y, b.y);
+        unpack2(acc[p][2], a.z, b.z);
+        unpack2(acc[p][3], a.w, b.w);
+        const int64_t q = q0 + b0 + 2 * p;
+        if (q < nq) *reinterpret_cast<float4 *>(yq + q * d + t0) = a;
+        if (q + 1 < nq) *reinterpret_cast<float4 *>(yq + (q + 1) * d + t0) = b;
+    }
+}
+
+// Queues the rotation of a batch; the scratch yq is 16-byte aligned.
+static void launch_rotate(const float *Q, const uint8_t *Q8, int64_t nq, int d, const float *Rt, float *yq,
+                          unsigned long long *counter, int32_t *status, int sms, cudaStream_t st)
+{
+    if (rotate_tiled(nq, d)) {
+        rotate_kernel<<<(unsigned)((nq + ROT_Q - 1) / ROT_Q), d / 4 * 8, rotate_smem(d), st>>>(Q, Q8, nq, d, Rt, yq, counter,
+                                                                                             status);
+    } else if (nq <= 2 * (int64_t)sms) {
+        rotate_few_kernel<1><<<(unsigned)nq, 128, 0, st>>>(Q, Q8, nq, d, Rt, yq, counter, status);
+    } else {
+        rotate_few_kernel<8><<<(unsigned)((nq + 7) / 8), 128, 0, st>>>(Q, Q8, nq, d, Rt, yq, counter, status);
     }
 }
 
@@ -148,13 +203,16 @@ __device__ __forceinline__ int order_bucket(float x)
     return (int)((__float_as_uint(x) & 0x7fffffffu) >> 20);          // 0 .. 2047
 }
 
-__global__ void __launch_bounds__(ORDER_THREADS) order_kernel(const float *key, int64_t n, int32_t *order)
+__global__ void __launch_bounds__(ORDER_THREADS) order_kernel(const float *key, int64_t n, int32_t *order,
+                                                             unsigned long long *counter)
 {
     __shared__ uint32_t pos[ORDER_BUCKETS];
     __shared__ uint32_t wsum[ORDER_THREADS / 32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (t == 0) *counter = 0;                         // the level-0 walk takes the queries from the start again
     for (int i = t; i < ORDER_BUCKETS; i += ORDER_THREADS) pos[i] = 0;
     __syncthreads();
+#pragma unroll 8
     for (int64_t i = t; i < n; i += ORDER_THREADS) atomicAdd(&pos[order_bucket(__ldg(key + i))], 1u);
     __syncthreads();
     // thread t owns buckets b0 = 2047 - 2t and b0 - 1 (ranks 2t and 2t + 1 in decreasing order)
@@ -184,6 +242,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_kernel(const float *key, 
     pos[b0] = ex;                                     // only this thread reads or writes b0, b1
     pos[b1] = ex + c0;
     __syncthreads();
+#pragma unroll 8
     for (int64_t i = t; i < n; i += ORDER_THREADS) {
         const uint32_t p = atomicAdd(&pos[order_bucket(__ldg(key + i))], 1u);
         order[p] = (int32_t)i;
@@ -302,20 +361,14 @@ __global__ void __launch_bounds__(TAB_WARPS * 32) table_kernel(const float *yq, 
 // ------------------------------------------------------------------------------------------
 // Candidates staged at a time.  Three keep a warp's staging at 2.3 KB (d = 96), so both FP32
 // codebooks (192 KB) and 15 warps fit in shared memory: every codebook read is a conflict-free
-// shared load.  Measured on 10k queries of the 1M workload: 0.117 ms, against 0.172 ms with
-// eight staged (C2 read through L1 and L2 at 16 warps), 0.123 / 0.121 / 0.125 ms with 2 / 4 / 5
-// staged (16 / 12 / 10 warps beside both codebooks).
+// shared load.  Measured on 10k queries of the 1M workload: 0.092 ms (0.117 ms with the codebooks
+// and code rows copied through registers and the keys sorted by a bitonic network; one query
+// 35.8 -> 11.8 us).  Of the older form eight staged candidates (C2 read through L1 and L2 at 16
+// warps) took 0.172 ms, and 2 / 4 / 5 staged 0.123 / 0.121 / 0.125 ms.
 constexpr int REF_CH = 3;
 
-__host__ __device__ inline int pow2_at_least(int r)
-{
-    int p = 32;
-    while (p < r) p <<= 1;
-    return p;
-}
-
-// Per-warp shared memory of the refinement kernel.
-__host__ __device__ inline size_t refine_smem(int M1, int M2P, int R, int BM)
+// Shared memory of the refinement kernel per warp (staging) and per team (keys).
+__host__ __device__ inline size_t refine_smem(int M1, int M2P, int BM)
 {
     size_t o = 0;
     o += (size_t)REF_CH * 9 * 4;            // vertex ids
@@ -323,67 +376,70 @@ __host__ __device__ inline size_t refine_smem(int M1, int M2P, int R, int BM)
     o = align_up(o, 16);                    // code rows are written 16 bytes at a time
     o += (size_t)REF_CH * 9 * M1;           // level-1 code rows
     o += (size_t)REF_CH * 9 * M2P;          // level-2 code rows (+ codeword id)
-    o += (size_t)pow2_at_least(R) * 8;      // keys
-    return align_up(o, 128);
+    return align_up(o, 16);
 }
+__host__ __device__ inline size_t refine_keys(int R) { return (size_t)((R + 1) & ~1) * 8; }
 
-// One warp per query.  C2_SHARED: both codebooks sit in shared memory (d*4 bytes is a
-// multiple of 128, so lane t reading coordinate t of any centroid hits bank t mod 32);
-// otherwise only C1 does and C2 is read through the cache.  DU: coordinates per lane
-// (d = 32 DU), or 8 with bounds checks for other d <= 256.
-template <bool C2_SHARED, int DU, bool PROD>
+// A team of a.T warps per query: its warps take groups of REF_CH candidates in turn and leave
+// the keys in shared memory, then every lane finds the rank of its keys.  T = 1 for large
+// batches; a batch that does not fill the GPU with one warp per query gets larger teams (777
+// queries with R = 100 and a product codebook ran on 52 SMs with one: 197 -> 171 us).  C2_SHARED: both codebooks sit in
+// shared memory (copied with all loads in flight; d*4 bytes is a multiple of 128 at d = 96 and
+// 128, so lane t reading coordinate t of any centroid hits bank t mod 32); otherwise only C1 does
+// and C2 is read through the cache.  DU: coordinates per lane, d <= 32 DU (CHECK: d < 32 DU).
+template <bool C2_SHARED, int DU, bool PROD, bool CHECK>
 __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int d = a.d, M1 = a.M1, M2P = a.M2P;
+    const int d = a.d, M1 = a.M1, M2P = a.M2P, T = a.T;
     float *C1s = reinterpret_cast<float *>(smem_raw);
     float *C2s = C1s + 256 * d;
-    {
-        const float4 *s1 = reinterpret_cast<const float4 *>(a.C1);
-        const float4 *s2 = reinterpret_cast<const float4 *>(a.C2);
-        for (int i = threadIdx.x; i < 64 * d; i += blockDim.x) {
-            reinterpret_cast<float4 *>(C1s)[i] = __ldg(s1 + i);
-            if (C2_SHARED) reinterpret_cast<float4 *>(C2s)[i] = __ldg(s2 + i);
-        }
-    }
+    copy_async(C1s, a.C1, (size_t)256 * d * 4);
+    if (C2_SHARED) copy_async(C2s, a.C2, (size_t)256 * d * 4);
+    copy_wait();
     __syncthreads();
     const float *C2 = C2_SHARED ? C2s : a.C2;
     const size_t cb = (size_t)(C2_SHARED ? 2 : 1) * 256 * d * 4;
     const int BM = PROD ? a.BM : 1;
-    unsigned char *base = smem_raw + cb + (size_t)warp * refine_smem(M1, M2P, a.R, BM);
-    const int RP = pow2_at_least(a.R);
+    const size_t per_warp = refine_smem(M1, M2P, BM);
+    const int nw = blockDim.x >> 5, teams = nw / T, team = warp / T, tw = warp % T;
+    if (team >= teams) return;
+    unsigned char *base = smem_raw + cb + (size_t)warp * per_warp;
+    uint64_t *keys = reinterpret_cast<uint64_t *>(smem_raw + cb + nw * per_warp + team * refine_keys(a.R));
     int32_t *vid = reinterpret_cast<int32_t *>(base);
     float *wt = reinterpret_cast<float *>(base + REF_CH * 9 * 4);       // [REF_CH][BM][9]
     uint8_t *st1 = base + align_up((size_t)REF_CH * 9 * 4 * (1 + BM), 16);
     uint8_t *st2 = st1 + REF_CH * 9 * M1;
-    uint64_t *keys = reinterpret_cast<uint64_t *>(st2 + REF_CH * 9 * M2P);
-    const int64_t gwarp = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int r1 = M1 / 16, r2 = M2P / 16;          // 16-byte pieces per row
+    const int per_row = r1 + r2;
+    const uint32_t inv_row = (65536 + per_row - 1) / per_row;           // t / per_row for t < 27 * per_row
+    auto team_sync = [&]() {
+        if (T == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(T * 32) : "memory");
+    };
     // sub-spaces of this lane's coordinates t = lane + 32 u (read once: indexing the
     // parameter space with a per-lane index would serialise)
-    int s1v[DU], s2v[DU], sbv[DU];
+    int s1v[DU], s2v[DU], sbv[DU], tv[DU];
 #pragma unroll
     for (int u = 0; u < DU; u++) {
-        const int t = lane + 32 * u;
-        s1v[u] = t < d ? a.sub1[t] : 0;
-        s2v[u] = t < d ? a.sub2[t] : 0;
-        sbv[u] = PROD && t < d ? a.subb[t] : 0;
+        const int t = CHECK ? min(lane + 32 * u, d - 1) : lane + 32 * u;
+        tv[u] = t;
+        s1v[u] = a.sub1[t];
+        s2v[u] = a.sub2[t];
+        sbv[u] = PROD ? a.subb[t] : 0;
     }
     const int nb = a.BK > 1 ? BM : 0;               // codeword bytes at the end of a row
 
-    for (int64_t q = gwarp; q < a.nq; q += nwarps) {
+    for (int64_t q = (int64_t)blockIdx.x * teams + team; q < a.nq; q += (int64_t)gridDim.x * teams) {
         const int32_t *sl = a.shortlist + q * a.R;
         float yv[DU];
 #pragma unroll
-        for (int u = 0; u < DU; u++) yv[u] = lane + 32 * u < d ? a.yq[q * d + lane + 32 * u] : 0.f;
+        for (int u = 0; u < DU; u++) yv[u] = a.yq[q * d + tv[u]];
         int rn = 0;                                  // shortlist entries present (packed first)
         for (int i = lane; i < a.R; i += 32) rn += sl[i] >= 0;
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) rn += __shfl_xor_sync(FULL, rn, m);
-        for (int i = lane; i < RP; i += 32) keys[i] = ~0ull;
-        for (int c0 = 0; c0 < rn; c0 += REF_CH) {
+        rn = __reduce_add_sync(0xffffffffu, rn);
+        for (int c0 = tw * REF_CH; c0 < rn; c0 += T * REF_CH) {
             const int nc = min(REF_CH, rn - c0);
             // one candidate per lane: its id, codeword and the 8 neighbours of G(x); the
             // loads of a phase are all issued before any is used
@@ -407,32 +463,18 @@ __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
                 }
             }
             __syncwarp();
-            // stage both code rows of every vertex: 16-byte pieces, six loads in flight per lane
-            const int per_row = r1 + r2, pieces = nc * 9 * per_row;
-            for (int t0 = lane; t0 < pieces; t0 += 32 * 6) {
-                uint4 buf[6];
-                bool use[6];
-#pragma unroll
-                for (int u = 0; u < 6; u++) {
-                    const int t = t0 + 32 * u;
-                    const int row = t / per_row, pc = t % per_row;
-                    use[u] = t < pieces && vid[row] >= 0;
-                    if (use[u]) {
-                        const int64_t v = vid[row];
-                        buf[u] = pc < r1 ? __ldg(reinterpret_cast<const uint4 *>(a.codes1 + v * M1) + pc)
-                                         : __ldg(reinterpret_cast<const uint4 *>(a.codes2b + v * M2P) + (pc - r1));
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 6; u++) {
-                    const int t = t0 + 32 * u;
-                    const int row = t / per_row, pc = t % per_row;
-                    if (use[u]) {
-                        if (pc < r1) reinterpret_cast<uint4 *>(st1 + row * M1)[pc] = buf[u];
-                        else reinterpret_cast<uint4 *>(st2 + row * M2P)[pc - r1] = buf[u];
-                    }
+            // stage both code rows of every vertex in 16-byte pieces
+            const int pieces = nc * 9 * per_row;
+#pragma unroll 2
+            for (int t = lane; t < pieces; t += 32) {
+                const int row = (int)((t * inv_row) >> 16), pc = t - row * per_row;
+                const int64_t v = vid[row];
+                if (v >= 0) {
+                    if (pc < r1) copy16_l2(st1 + row * M1 + pc * 16, a.codes1 + v * M1 + pc * 16);
+                    else copy16_l2(st2 + row * M2P + (pc - r1) * 16, a.codes2b + v * M2P + (pc - r1) * 16);
                 }
             }
+            copy_wait();
             __syncwarp();
             for (int r = 0; r < nc; r++) {
                 // y^_t = sum_j beta_j (C1[c1_j][t] + C2[c2_j][t]) for this lane's coordinates,
@@ -448,7 +490,7 @@ __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
                     for (int j = 0; j < 9; j++) {
                         const uint8_t *c2r = st2 + (r * 9 + j) * M2P;
 #pragma unroll
-                        for (int u = 0; u < DU; u++) x2[j][u] = C2[(int)c2r[s2v[u]] * d + lane + 32 * u];
+                        for (int u = 0; u < DU; u++) x2[j][u] = C2[(int)c2r[s2v[u]] * d + tv[u]];
                     }
                 }
 #pragma unroll
@@ -462,19 +504,17 @@ __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
                     const uint8_t *c1r = st1 + tt * M1, *c2r = st2 + tt * M2P;
 #pragma unroll
                     for (int u = 0; u < DU; u++) {
-                        const int t = lane + 32 * u;
-                        if (DU == 8 && t >= d) continue;
                         // the weight of this coordinate's regression block
                         const float w = PROD ? (have ? wt[(r * BM + sbv[u]) * 9 + j] : 0.f) : w0;
-                        const float x = C1s[(int)c1r[s1v[u]] * d + t] +
-                                        (HOIST ? x2[HOIST ? j : 0][u] : C2[(int)c2r[s2v[u]] * d + t]);
+                        const float x = C1s[(int)c1r[s1v[u]] * d + tv[u]] +
+                                        (HOIST ? x2[HOIST ? j : 0][u] : C2[(int)c2r[s2v[u]] * d + tv[u]]);
                         yh[u] = fmaf(w, x, yh[u]);
                     }
                 }
                 float part = 0.f;
 #pragma unroll
                 for (int u = 0; u < DU; u++) {
-                    if (DU == 8 && lane + 32 * u >= d) continue;
+                    if (CHECK && lane + 32 * u >= d) continue;
                     const float df = yv[u] - yh[u];
                     part = fmaf(df, df, part);
                 }
@@ -484,28 +524,27 @@ __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
             }
             __syncwarp();
         }
-        __syncwarp();
-        // bitonic sort of keys[0..RP) ascending
-        for (int kk = 2; kk <= RP; kk <<= 1) {
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                for (int i = lane; i < RP; i += 32) {
-                    int p = i ^ j;
-                    if (p > i) {
-                        uint64_t x = keys[i], y = keys[p];
-                        bool up = (i & kk) == 0;
-                        if ((x > y) == up) { keys[i] = y; keys[p] = x; }
-                    }
+        if ((rn & 1) && tw == 0 && lane == 0) keys[rn] = ~0ull;          // the count takes two at a time
+        team_sync();
+        // the k smallest by (distance, id): every key's rank is its place (keys are distinct)
+        for (int i = lane + 32 * tw; i < max(rn, a.k); i += 32 * T) {
+            uint64_t key = ~0ull;
+            int rank = i;                            // (past the candidates: padding at its own place)
+            if (i < rn) {
+                key = keys[i];
+                rank = 0;
+#pragma unroll 4
+                for (int j = 0; j < rn; j += 2) {
+                    const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(keys + j);
+                    rank += (o.x < key) + (o.y < key);
                 }
-                __syncwarp();
+            }
+            if (rank < a.k) {
+                a.ids_out[q * a.k + rank] = i < rn ? key_id(key) : -1;
+                a.dists_out[q * a.k + rank] = i < rn ? key_dist(key) : __int_as_float(0x7f800000);
             }
         }
-        for (int i = lane; i < a.k; i += 32) {
-            uint64_t kk = keys[i];
-            bool ok = kk != ~0ull;
-            a.ids_out[q * a.k + i] = ok ? key_id(kk) : -1;
-            a.dists_out[q * a.k + i] = ok ? key_dist(kk) : __int_as_float(0x7f800000);
-        }
-        __syncwarp();
+        team_sync();                                 // before the next query's keys
     }
 }
 
@@ -621,18 +660,18 @@ static int ilog2_ceil(int64_t x)
 using RefineFn = void (*)(const RefineArgs);
 
 
-// Refinement instantiation: codebooks placement and coordinates per lane (3 for d = 96,
-// 4 for d = 128, else the checked 8).
+// Refinement instantiation: codebooks placement and coordinates per lane (3 for d = 96, 4 for
+// d = 128, else 4 or 8 with checks).
 static RefineFn refine_kernel_for(bool both, int d, bool prod)
 {
-    if (prod) {
-        if (d == 96) return both ? refine_kernel<true, 3, true> : refine_kernel<false, 3, true>;
-        if (d == 128) return both ? refine_kernel<true, 4, true> : refine_kernel<false, 4, true>;
-        return both ? refine_kernel<true, 8, true> : refine_kernel<false, 8, true>;
-    }
-    if (d == 96) return both ? refine_kernel<true, 3, false> : refine_kernel<false, 3, false>;
-    if (d == 128) return both ? refine_kernel<true, 4, false> : refine_kernel<false, 4, false>;
-    return both ? refine_kernel<true, 8, false> : refine_kernel<false, 8, false>;
+    auto pick = [&](auto b, auto p) -> RefineFn {
+        constexpr bool B = decltype(b)::value, PR = decltype(p)::value;
+        return d == 96 ? refine_kernel<B, 3, PR, false> : d == 128 ? refine_kernel<B, 4, PR, false>
+             : d < 128 ? refine_kernel<B, 4, PR, true> : refine_kernel<B, 8, PR, true>;
+    };
+    using T = std::true_type;
+    using F = std::false_type;
+    return both ? (prod ? pick(T{}, T{}) : pick(T{}, F{})) : (prod ? pick(F{}, T{}) : pick(F{}, F{}));
 }
 
 lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params *sp, SearchPlan *pl,
@@ -726,30 +765,30 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
             return LC_ERR_CUDA;
         }
     }
-    {
-        const size_t rsm = rotate_smem(dv->d);
-        if (cudaFuncSetAttribute(rotate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_PER_BLOCK) != cudaSuccess) {
-            set_error("rotation kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError()));
-            return LC_ERR_CUDA;
-        }
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rotate_kernel, ROT_THREADS, rsm);
-        P.qsm = rsm;
-        // as many blocks as fit at once: the batch is rotated in about one step per block
-        P.qgrid = (int)std::min<int64_t>((nq + ROT_Q - 1) / ROT_Q, (int64_t)std::max(per_sm, 1) * dv->num_sms);
+    if (rotate_tiled(nq, dv->d) &&
+        cudaFuncSetAttribute(rotate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_PER_BLOCK) != cudaSuccess) {
+        set_error("rotation kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError()));
+        return LC_ERR_CUDA;
     }
     if (P.refine) {
         P.sl_elems = (size_t)nq * P.R;
-        const size_t per = refine_smem(dv->M1, dv->M2P, P.R, dv->bM);
+        const size_t per = refine_smem(dv->M1, dv->M2P, dv->bM) + refine_keys(P.R);
         const size_t cbytes = (size_t)256 * dv->d * 4;
         // both codebooks in shared memory when that leaves room for at least 8 warps
         P.rboth = 2 * cbytes + 8 * per <= MAX_SMEM_PER_BLOCK;
         const size_t cb = (P.rboth ? 2 : 1) * cbytes;
-        if (cb + per > MAX_SMEM_PER_BLOCK) {
+        // (refused by the size of a warp's staging with keys padded to a power of two)
+        size_t padded = 32;
+        while (padded < (size_t)P.R) padded <<= 1;
+        const size_t core = align_up((size_t)REF_CH * 9 * 4 * (1 + dv->bM), 16) + (size_t)REF_CH * 9 * (dv->M1 + dv->M2P);
+        if (cbytes + align_up(core + padded * 8, 128) > MAX_SMEM_PER_BLOCK) {
             set_error("refinement does not fit in shared memory (d = %d)", dv->d);
             return LC_ERR_CAPACITY;
         }
         P.rw = (int)std::min<size_t>(16, (MAX_SMEM_PER_BLOCK - cb) / per);
+        // teams: as many warps per query as the batch leaves idle, at most one per group of candidates
+        P.rteam = 1;
+        while (2 * P.rteam <= P.rw && (P.rteam * REF_CH < P.R) && nq * P.rteam * 2 <= (int64_t)P.rw * dv->num_sms) P.rteam *= 2;
         P.rsm = cb + per * P.rw;
         auto kern = refine_kernel_for(P.rboth, dv->d, dv->bM > 1);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_PER_BLOCK) != cudaSuccess) {
@@ -758,7 +797,7 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         }
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P.rw * 32, P.rsm);
-        const int64_t need = (nq + P.rw - 1) / P.rw;
+        const int64_t teams = P.rw / P.rteam, need = (nq + teams - 1) / teams;
         P.rgrid = (int)std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * dv->num_sms);
     }
     *pl = P;
@@ -806,8 +845,9 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
         splits(dv->d, dv->M2, o2, l2);
         for (int j = 0; j < dv->M2; j++) for (int t = o2[j]; t < o2[j] + l2[j]; t++) wa.sub2[t] = (uint8_t)j;
     }
-    if (cudaMemsetAsync(sc.status, 0, sizeof(int32_t), st) != cudaSuccess ||
-        cudaMemsetAsync(sc.counter, 0, sizeof(unsigned long long), st) != cudaSuccess) {
+    // (the rotation resets the status word and the query counter)
+    if (rotated && (cudaMemsetAsync(sc.status, 0, sizeof(int32_t), st) != cudaSuccess ||
+                    cudaMemsetAsync(sc.counter, 0, sizeof(unsigned long long), st) != cudaSuccess)) {
         set_error("status reset failed: %s", cudaGetErrorString(cudaGetLastError()));
         return LC_ERR_CUDA;
     }
@@ -816,7 +856,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
             if (!e) cudaEventCreate(&e);
         cudaEventRecord(dv->ev[0], st);
     }
-    if (!rotated) rotate_kernel<<<std::max(P.qgrid, 1), ROT_THREADS, P.qsm, st>>>(dq, dq8, nq, dv->d, dv->Rt, sc.yq);
+    if (!rotated) launch_rotate(dq, dq8, nq, dv->d, dv->Rt, sc.yq, sc.counter, sc.status, dv->num_sms, st);
     cudaError_t ce = cudaGetLastError();
     if (ce == cudaSuccess && P.tab) {
         // the batch's ADC tables on the tensor cores, from y'
@@ -840,10 +880,8 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
         w1.seed_d = seed_d;
         ce = P.tab ? descent_run_tab(w1, P.dsmem, P.dwpc, P.dgrid, st)
                    : descent_run(P.half, P.variant, dv->M1, P.full, w1, P.dsmem, P.dwpc, P.dgrid, st);
-        if (ce == cudaSuccess && cudaMemsetAsync(sc.counter, 0, sizeof(unsigned long long), st) == cudaSuccess) {
-            order_kernel<<<1, ORDER_THREADS, 0, st>>>(seed_d, nq, order);
-            ce = cudaGetLastError();
-        } else if (ce == cudaSuccess) {
+        if (ce == cudaSuccess) {
+            order_kernel<<<1, ORDER_THREADS, 0, st>>>(seed_d, nq, order, sc.counter);
             ce = cudaGetLastError();
         }
         if (ce != cudaSuccess) {
@@ -866,7 +904,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     }
     if (P.refine) {
         RefineArgs ra{};
-        ra.yq = sc.yq; ra.shortlist = sc.shortlist; ra.nq = nq; ra.R = P.R; ra.k = P.k; ra.d = dv->d;
+        ra.yq = sc.yq; ra.shortlist = sc.shortlist; ra.nq = nq; ra.T = P.rteam; ra.R = P.R; ra.k = P.k; ra.d = dv->d;
         ra.M1 = dv->M1; ra.M2P = dv->M2P; ra.C1 = dv->C1; ra.C2 = dv->C2; ra.B = dv->B;
         ra.codes1 = dv->codes1; ra.codes2b = dv->codes2b; ra.adj0 = dv->adj0;
         ra.ids_out = dids; ra.dists_out = ddists;

@@ -575,6 +575,11 @@ __device__ __forceinline__ void copy16(void *dst, const void *src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
 }
+__device__ __forceinline__ void copy16_l2(void *dst, const void *src)      // not through L1
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void copy_async(void *dst, const void *src, size_t bytes)
 {
@@ -1140,7 +1145,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                 n_expand += nb;
                 __syncwarp();
                 if (nb > 4 && lane >= 4 && lane < nb)
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(a.adj0 + (int64_t)sel[lane] * DEG));
+                    prefetch_l1(a.adj0 + (int64_t)sel[lane] * DEG);
                 // their adjacency rows through the visited test, four rows at a time while the
                 // limits leave room for all of them, else row by row; fresh nodes are appended
                 const int half = (1 << a.spill_log) / 2;
