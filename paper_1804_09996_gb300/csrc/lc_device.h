@@ -106,6 +106,9 @@ struct VisitTab {
     uint32_t mul, bytes;           // multiplier, bytes of the buckets
 };
 
+// The walk's element types: FP32 or FP16 codebook, per-query tables.
+enum WalkForm { WALK_F32, WALK_F16, WALK_TAB };
+
 // Launch configuration of one search and the scratch it needs.
 struct SearchPlan {
     int k = 0, efp = 0, R = 0, beam = 1, tcap = 0, hash_log = 0, spill_log = 0, variant = 0;
@@ -125,6 +128,7 @@ struct SearchPlan {
     VisitTab vt{};                       // visited set in shared memory
     int64_t spill_tables = 0;            // global visited tables
     size_t yq_elems = 0, sl_elems = 0, spill_elems = 0, ord_elems = 0;
+    WalkForm form() const { return tab ? WALK_TAB : half ? WALK_F16 : WALK_F32; }
 };
 
 // Device scratch of one search in flight.

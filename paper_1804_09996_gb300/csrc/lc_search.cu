@@ -725,12 +725,10 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     cudaError_t ce;
     if (!fits) {
         ce = cudaErrorInvalidConfiguration;
-    } else if (P.tab) {
-        P.tab_elems = (size_t)nq * 256 * TAB_M1;
-        ce = walk_config_tab(wa, P.per_warp, dv->num_sms, sp->warps, &P.wpc, &P.grid, &P.smem);
     } else {
-        ce = walk_config(P.half, P.variant, dv->M1, P.full, wa, P.per_warp, dv->num_sms, sp->warps, &P.wpc, &P.grid,
-                         &P.smem);
+        P.tab_elems = P.tab ? (size_t)nq * 256 * TAB_M1 : 0;
+        wa.beam = P.beam;
+        ce = walk_config(P.form(), P.variant, dv->M1, P.full, wa, P.per_warp, dv->num_sms, sp->warps, &P.wpc, &P.grid, &P.smem);
     }
     if (ce == cudaErrorInvalidConfiguration) {
         set_error("search too wide for shared memory (%zu B per query in flight next to a %zu B codebook); "
@@ -758,8 +756,7 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         wd.nq = nq;
         wd.d = dv->d;
         wd.M2P = dv->M2P;
-        ce = P.tab ? descent_config_tab(wd, dv->num_sms, &P.dwpc, &P.dgrid, &P.dsmem)
-                   : descent_config(P.half, P.variant, dv->M1, P.full, wd, dv->num_sms, &P.dwpc, &P.dgrid, &P.dsmem);
+        ce = descent_config(P.form(), P.variant, dv->M1, P.full, wd, dv->num_sms, &P.dwpc, &P.dgrid, &P.dsmem);
         if (ce != cudaSuccess) {
             set_error("descent kernel configuration failed: %s", cudaGetErrorString(ce));
             return LC_ERR_CUDA;
@@ -878,8 +875,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
         w1.seed = seed;
         w1.seed_up = seed_up;
         w1.seed_d = seed_d;
-        ce = P.tab ? descent_run_tab(w1, P.dsmem, P.dwpc, P.dgrid, st)
-                   : descent_run(P.half, P.variant, dv->M1, P.full, w1, P.dsmem, P.dwpc, P.dgrid, st);
+        ce = descent_run(P.form(), P.variant, dv->M1, P.full, w1, P.dsmem, P.dwpc, P.dgrid, st);
         if (ce == cudaSuccess) {
             order_kernel<<<1, ORDER_THREADS, 0, st>>>(seed_d, nq, order, sc.counter);
             ce = cudaGetLastError();
@@ -895,8 +891,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
         wa.seed_d = seed_d;
     }
     if (profile) cudaEventRecord(dv->ev[4], st);
-    ce = P.tab ? walk_run_tab(wa, P.smem, P.wpc, P.grid, st)
-               : walk_run(P.half, P.variant, dv->M1, P.full, wa, P.smem, P.wpc, P.grid, st);
+    ce = walk_run(P.form(), P.variant, dv->M1, P.full, wa, P.smem, P.wpc, P.grid, st);
     if (profile) cudaEventRecord(dv->ev[1], st);
     if (ce != cudaSuccess) {
         set_error("walk kernel launch failed: %s", cudaGetErrorString(ce));
@@ -1184,7 +1179,7 @@ lc_status search_walk_noalloc(lc_index *ix, const float *q, int64_t nq, int k, i
     // every warp in flight owns one spill table of the array
     const size_t slots = NOALLOC_SPILL_BYTES / ((size_t)4 << wa.spill_log);
     const int want = (int)std::max<size_t>(1, slots / std::max(1, dv->num_sms));     // all SMs before more walks on each
-    ce = walk_config(false, variant, dv->M1, false, wa, per_warp, dv->num_sms, want, &wpc, &grid, &smem);
+    ce = walk_config(WALK_F32, variant, dv->M1, false, wa, per_warp, dv->num_sms, want, &wpc, &grid, &smem);
     if (ce != cudaSuccess) {
         set_error("walk kernel configuration failed: %s", cudaGetErrorString(ce));
         return ce == cudaErrorInvalidConfiguration ? LC_ERR_CAPACITY : LC_ERR_CUDA;
@@ -1197,7 +1192,7 @@ lc_status search_walk_noalloc(lc_index *ix, const float *q, int64_t nq, int k, i
         return LC_ERR_CUDA;
     }
     wa.spill_tables = (int64_t)grid * wpc;
-    ce = walk_run(false, variant, dv->M1, false, wa, smem, wpc, grid, st);
+    ce = walk_run(WALK_F32, variant, dv->M1, false, wa, smem, wpc, grid, st);
     if (ce != cudaSuccess) {
         set_error("walk kernel launch failed: %s", cudaGetErrorString(ce));
         return LC_ERR_CUDA;
@@ -1399,7 +1394,7 @@ lc_status plan_create(lc_index *ix, int64_t nq_max, const lc_search_params *sp, 
     // find the two kernel nodes whose batch size a smaller call updates
     // (the rotation and, in the table form, the table launch keep the largest batch: their
     // extra rows are computed and not read)
-    const void *wf = P.tab ? walk_fn_tab() : walk_fn(P.half, P.variant, dv->M1, P.full);
+    const void *wf = walk_fn(P.form(), P.variant, dv->M1, P.full, P.beam > 1);
     const void *rf = P.refine ? (const void *)refine_kernel_for(P.rboth, d, dv->bM > 1) : nullptr;
     size_t nn = 0;
     cudaGraphGetNodes(pl->graph, nullptr, &nn);

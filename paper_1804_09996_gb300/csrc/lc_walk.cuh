@@ -611,10 +611,11 @@ __device__ __forceinline__ void stage_codes(uint8_t *stage, int rows, const uint
     __syncwarp();
 }
 
-// Walk distances of nf staged nodes (1 <= nf <= 32), block by block, two blocks at once where
-// there are two (their chains of shared-memory reads and shuffles overlap).  Returns the total of
-// node chunk_slot(lane) (undefined from nf on).
-template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
+// Walk distances of nf staged nodes (1 <= nf <= 32), block by block; PAIR: two blocks at once
+// where there are two (their chains of shared-memory reads and shuffles overlap: 2 % for the
+// batched walk, whose chunks are full; for the plain one the extra code costs more).  Returns the
+// total of node chunk_slot(lane) (undefined from nf on).
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool PAIR>
 __device__ __forceinline__ float score_staged(const CT *C1s, const uint8_t *stage, const uint8_t *stage2, int nf, int d,
                                               const LaneGeo<M1, D1> &g, int lane, const CT *C2, int M2P)
 {
@@ -626,7 +627,6 @@ __device__ __forceinline__ float score_staged(const CT *C1s, const uint8_t *stag
         if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, TAB, false>(C1s, st, st2, d, g, lane, C2, M2P, v);
         else block_terms<M1, D1, CT, FQ, TAB, true>(C1s, st, st2, d, g, lane, C2, M2P, v);
     };
-    constexpr bool PAIR = !FQ && D1 > 0;
 #pragma unroll 1
     for (int b = 0; b * SB < nf; b += PAIR ? 2 : 1) {
         float v[8];
@@ -930,14 +930,16 @@ __device__ __forceinline__ int members_below(const uint64_t *W, int wn, uint64_t
 // places not taken hold the members in order, so from the last 32 places down every place finds
 // its member from the number of candidates placed below it (one OR over the warp), and no member
 // searches; members only move up, so the places below are still the old ones.  Up to 32
-// candidates (nearly every step) stay in registers; else place[] keeps their places.
+// candidates (nearly every step; always unless MANY) stay in registers; else place[] keeps their
+// places.
+template <bool MANY>
 __device__ __forceinline__ int merge_step(uint64_t *W, int wn, int efp, uint64_t *cand, int nc, int32_t *place, int lane,
                                           int *first_new)
 {
     const int wn2 = min(efp, wn + nc);
     if (lane < 3) cand[nc + lane] = ~0ull;               // the count below takes four at a time
     __syncwarp();
-    const bool one = nc <= 32;
+    const bool one = !MANY || nc <= 32;
     int at = 0x7fffffff, lowest = 0x7fffffff;
     uint64_t k = 0;
 #pragma unroll 1
@@ -1013,7 +1015,11 @@ __device__ __forceinline__ void load_codebooks(const WalkArgs &a, unsigned char 
 
 // TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
 // [256][M1] (FP16, built by table_kernel) in shared memory and scores nodes by table lookups.
-template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
+// BATCH: beam > 1.  The plain walk is an instantiation of its own: it visits one row and merges at
+// most 32 candidates a step, and the step's code has to stay small (the instruction cache bounds
+// it: with the code for four rows beside its own the plain walk of 10k queries took 908 and not
+// 853 us).
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
 __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1033,7 +1039,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
     uint64_t *cand = reinterpret_cast<uint64_t *>(base + L.cand);
     int32_t *sel = reinterpret_cast<int32_t *>(base + L.sel);
     int32_t *slot = reinterpret_cast<int32_t *>(base + L.slot);
-    const int SR = stage_rows(M1 + (FQ ? a.M2P : 0), a.beam, a.vt.tag);
+    const int SR = BATCH ? stage_rows(M1 + (FQ ? a.M2P : 0), a.beam, a.vt.tag) : 32;
     const int64_t gwarp = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
     Visited V;
     V.tab = base + L.hash;
@@ -1098,7 +1104,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
         int wn = 1;
         bool failed = false;
         int scan_from = 0;                 // every member of W before it is expanded
-        const int B = a.beam;              // level-0 expansions per step; 1 = the plain walk
+        const int B = BATCH ? a.beam : 1;  // level-0 expansions per step
         if (a.mode == 2) {
             // level 0 from the entry node the descent launch recorded (as at its end below)
             cur = __ldg(a.seed + q);
@@ -1144,14 +1150,14 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                 if (nb == 0) break;
                 n_expand += nb;
                 __syncwarp();
-                if (nb > 4 && lane >= 4 && lane < nb)
+                if (BATCH && nb > 4 && lane >= 4 && lane < nb)
                     prefetch_l1(a.adj0 + (int64_t)sel[lane] * DEG);
                 // their adjacency rows through the visited test, four rows at a time while the
                 // limits leave room for all of them, else row by row; fresh nodes are appended
                 const int half = (1 << a.spill_log) / 2;
 #pragma unroll 1
                 for (int r0 = 0; r0 < nb;) {
-                    int cnt = min(4, nb - r0);
+                    int cnt = BATCH ? min(4, nb - r0) : 1;
                     if (V.spilled ? V.scount + 32 * cnt > half : V.hcount + 32 * cnt > shared_visited_cap(H)) {
                         cnt = 1;
                         if (!V.spilled && V.hcount + 32 > shared_visited_cap(H)) {
@@ -1167,7 +1173,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                     if (!a.vt.tag) {
                         nf = visit_rows_ids(V.tab_s, V.own_s, a.vt.bb, V.spill, a.spill_log, V.spilled, a.adj0, sel + r0,
                                             cnt, slot, ns, lane);
-                    } else if (cnt == 1) {
+                    } else if constexpr (!BATCH) {
                         const int32_t ev[1] = {__ldg(a.adj0 + (int64_t)sel[r0] * DEG + lane)};
                         nf = visit_rows<true, 1>(V, a.vt, a.spill_log, ev, slot, ns, lane);
                     } else {
@@ -1193,11 +1199,11 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             const uint64_t wmax = phase == 2 && wn == efp ? W[wn - 1] : ~0ull;
             int nc = 0;
 #pragma unroll 1
-            for (int ch = 0; ch < ns; ch += 32) {
-                const int at = ch % SR;                  // place in the staging area
+            for (int ch = 0; ch < ns; ch += 32) {          // (once unless BATCH)
+                const int at = BATCH ? ch % SR : 0;                  // place in the staging area
                 if (at == 0) stage_codes<M1, FQ>(stage, SR, a.codes1, a.codes2b, a.M2P, slot + ch, min(SR, ns - ch), lane);
                 const int nf = min(32, ns - ch);
-                const float de = score_staged<M1, D1, CT, FQ, TAB>(C1s, stage + at * M1, stage + SR * M1 + at * a.M2P, nf, d, g,
+                const float de = score_staged<M1, D1, CT, FQ, TAB, BATCH && !FQ && (D1 > 0)>(C1s, stage + at * M1, stage + SR * M1 + at * a.M2P, nf, d, g,
                                                                    lane, C2, a.M2P);
                 const int32_t id = my_slot < nf ? slot[ch + my_slot] : -1;
                 if (phase < 2) {                         // at most 32 nodes here
@@ -1236,7 +1242,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                 }
             } else if (nc > 0) {
                 int first_new;
-                wn = merge_step(W, wn, efp, cand, nc, slot, lane, &first_new);
+                wn = merge_step<BATCH>(W, wn, efp, cand, nc, slot, lane, &first_new);
                 scan_from = min(scan_from, first_new & ~31);
                 __syncwarp();
             }
@@ -1337,7 +1343,7 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
             uint32_t bd = ~0u, bi = ~0u;
             if (ns > 0) {
                 stage_codes<M1, FQ>(stage, 32, a.codes1, a.codes2b, a.M2P, slot, ns, lane);
-                const float de = score_staged<M1, D1, CT, FQ, TAB>(T1, stage, stage + 32 * M1, ns, d, g, lane, C2, a.M2P);
+                const float de = score_staged<M1, D1, CT, FQ, TAB, !FQ && (D1 > 0)>(T1, stage, stage + 32 * M1, ns, d, g, lane, C2, a.M2P);
                 const int32_t id = my_slot < ns ? slot[my_slot] : -1;
                 warp_best(id >= 0 ? __float_as_uint(de) : ~0u, (uint32_t)id, &bd, &bi);
             }
@@ -1410,7 +1416,7 @@ static cudaError_t run_descent(const WalkArgs &wa, size_t smem, int wpc, int gri
 
 // Warps per CTA: as many as fit next to the codebook (at most MAX_WALK_WARPS, and at most
 // want if want > 0).
-template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
 static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num_sms, int want, int *wpc_out,
                                int *grid_out, size_t *smem_out)
 {
@@ -1423,11 +1429,11 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     size_t smem = c1 + smem_per_warp * wpc;
     // the attribute is an upper bound: set to the maximum, so plans made in any order (the
     // server plans at submission and launches later) all remain launchable
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<M1, D1, CT, FQ, TAB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)MAX_SMEM_PER_BLOCK);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<M1, D1, CT, FQ, TAB>, wpc * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, wpc * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     int64_t need = (wa.nq + wpc - 1) / wpc;
@@ -1437,72 +1443,85 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     return cudaSuccess;
 }
 
-template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
 static cudaError_t run_walk(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st)
 {
-    walk_kernel<M1, D1, CT, FQ, TAB><<<grid, wpc * 32, smem, st>>>(wa);
+    walk_kernel<M1, D1, CT, FQ, TAB, BATCH><<<grid, wpc * 32, smem, st>>>(wa);
     return cudaGetLastError();
 }
 
-
-// Per element type (lc_walk_f32.cu, lc_walk_f16.cu): launch shape, launch and kernel address
-// of the instantiation for a sub-space width variant, M1 and the full-decode flag.
-cudaError_t walk_config_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms, int want,
-                            int *wpc, int *grid, size_t *smem);
-cudaError_t walk_run_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                         cudaStream_t st);
-const void *walk_fn_f32(int variant, int M1, bool fq);
-cudaError_t walk_config_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms, int want,
-                            int *wpc, int *grid, size_t *smem);
-cudaError_t walk_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                         cudaStream_t st);
-const void *walk_fn_f16(int variant, int M1, bool fq);
-
-cudaError_t descent_config_f32(int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,
-                               size_t *smem);
-cudaError_t descent_run_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                            cudaStream_t st);
-cudaError_t descent_config_f16(int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,
-                               size_t *smem);
-cudaError_t descent_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                            cudaStream_t st);
-
-inline cudaError_t descent_config(bool half, int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc,
-                                  int *grid, size_t *smem)
+// Runs f(WalkShape<M1, D1, FQ>) for the instantiation of a sub-space width variant, M1 and the
+// full-decode flag.  The full walk exists for the uniform splits and, in FP32, for any split.
+template <typename CT, typename F>
+static auto by_shape(int variant, int M1, bool fq, F &&f) -> decltype(f(WalkShape<16, 6, false>{}))
 {
-    return half ? descent_config_f16(variant, M1, fq, wa, sms, wpc, grid, smem)
-                : descent_config_f32(variant, M1, fq, wa, sms, wpc, grid, smem);
-}
-inline cudaError_t descent_run(bool half, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc,
-                               int grid, cudaStream_t st)
-{
-    return half ? descent_run_f16(variant, M1, fq, wa, smem, wpc, grid, st)
-                : descent_run_f32(variant, M1, fq, wa, smem, wpc, grid, st);
+    if (fq) {
+        switch (variant) {
+        case 1: return f(WalkShape<16, 6, true>{});
+        case 2: return f(WalkShape<32, 3, true>{});
+        case 3: return f(WalkShape<64, 2, true>{});
+        default:
+            if constexpr (sizeof(CT) == 4)
+                return M1 == 16 ? f(WalkShape<16, 0, true>{}) : M1 == 32 ? f(WalkShape<32, 0, true>{})
+                                                               : f(WalkShape<64, 0, true>{});
+            else
+                return decltype(f(WalkShape<16, 6, false>{}))(cudaErrorInvalidValue);
+        }
+    }
+    switch (variant) {
+    case 1: return f(WalkShape<16, 6, false>{});
+    case 2: return f(WalkShape<32, 3, false>{});
+    case 3: return f(WalkShape<64, 2, false>{});
+    default: return M1 == 16 ? f(WalkShape<16, 0, false>{}) : M1 == 32 ? f(WalkShape<32, 0, false>{})
+                                                             : f(WalkShape<64, 0, false>{});
+    }
 }
 
-// The table form (LC_LUT_TABLE; M1 = 32 at d = 96): launch shape, launch, kernel address of
-// the walk, and the descent launch of an ordered search.
-cudaError_t walk_config_tab(const WalkArgs &wa, size_t per_warp, int sms, int want, int *wpc, int *grid, size_t *smem);
-cudaError_t walk_run_tab(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st);
-const void *walk_fn_tab();
-cudaError_t descent_config_tab(const WalkArgs &wa, int sms, int *wpc, int *grid, size_t *smem);
-cudaError_t descent_run_tab(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st);
+// Launch shape, launch and kernel address of the walk, launch shape and launch of the descent, per
+// codebook element type (lc_walk_f32.cu, lc_walk_f16.cu) and for the table form (LC_LUT_TABLE;
+// M1 = 32 at d = 96).  Which walk instantiation also depends on wa.beam (walk_fn: batch).
+#define WALK_ENTRIES(NAME)                                                                                                  \
+    cudaError_t walk_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms, int want,    \
+                                   int *wpc, int *grid, size_t *smem);                                                      \
+    cudaError_t walk_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,           \
+                                cudaStream_t st);                                                                           \
+    const void *walk_fn_##NAME(int variant, int M1, bool fq, bool batch);                                                   \
+    cudaError_t descent_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,       \
+                                      size_t *smem);                                                                        \
+    cudaError_t descent_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,        \
+                                   cudaStream_t st);
+WALK_ENTRIES(f32)
+WALK_ENTRIES(f16)
+WALK_ENTRIES(tab)
+#undef WALK_ENTRIES
 
-inline cudaError_t walk_config(bool half, int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms,
+// The same for the form of a search.
+inline cudaError_t walk_config(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms,
                                int want, int *wpc, int *grid, size_t *smem)
 {
-    return half ? walk_config_f16(variant, M1, fq, wa, per_warp, sms, want, wpc, grid, smem)
-                : walk_config_f32(variant, M1, fq, wa, per_warp, sms, want, wpc, grid, smem);
+    return (f == WALK_F32 ? walk_config_f32 : f == WALK_F16 ? walk_config_f16 : walk_config_tab)(variant, M1, fq, wa, per_warp,
+                                                                                              sms, want, wpc, grid, smem);
 }
-inline cudaError_t walk_run(bool half, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc,
-                            int grid, cudaStream_t st)
+inline cudaError_t walk_run(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
+                            cudaStream_t st)
 {
-    return half ? walk_run_f16(variant, M1, fq, wa, smem, wpc, grid, st)
-                : walk_run_f32(variant, M1, fq, wa, smem, wpc, grid, st);
+    return (f == WALK_F32 ? walk_run_f32 : f == WALK_F16 ? walk_run_f16 : walk_run_tab)(variant, M1, fq, wa, smem, wpc, grid, st);
 }
-inline const void *walk_fn(bool half, int variant, int M1, bool fq)
+inline const void *walk_fn(WalkForm f, int variant, int M1, bool fq, bool batch)
 {
-    return half ? walk_fn_f16(variant, M1, fq) : walk_fn_f32(variant, M1, fq);
+    return (f == WALK_F32 ? walk_fn_f32 : f == WALK_F16 ? walk_fn_f16 : walk_fn_tab)(variant, M1, fq, batch);
+}
+inline cudaError_t descent_config(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,
+                                  size_t *smem)
+{
+    return (f == WALK_F32 ? descent_config_f32 : f == WALK_F16 ? descent_config_f16 : descent_config_tab)(variant, M1, fq, wa,
+                                                                                                       sms, wpc, grid, smem);
+}
+inline cudaError_t descent_run(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
+                               cudaStream_t st)
+{
+    return (f == WALK_F32 ? descent_run_f32 : f == WALK_F16 ? descent_run_f16 : descent_run_tab)(variant, M1, fq, wa, smem, wpc,
+                                                                                              grid, st);
 }
 
 }  // namespace lc
