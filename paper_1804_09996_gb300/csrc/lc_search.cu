@@ -783,9 +783,15 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
             return LC_ERR_CAPACITY;
         }
         P.rw = (int)std::min<size_t>(16, (MAX_SMEM_PER_BLOCK - cb) / per);
-        // teams: as many warps per query as the batch leaves idle, at most one per group of candidates
-        P.rteam = 1;
-        while (2 * P.rteam <= P.rw && (P.rteam * REF_CH < P.R) && nq * P.rteam * 2 <= (int64_t)P.rw * dv->num_sms) P.rteam *= 2;
+        // teams: the number of warps per query that ends first, counted in candidates per warp: rounds
+        // of queries times the candidates of a team's busiest warp and its overhead (about two)
+        const int groups = (P.R + REF_CH - 1) / REF_CH;
+        int64_t best = INT64_MAX;
+        for (int t = 1; t <= std::min(P.rw, groups); t++) {
+            const int64_t per_round = (int64_t)(P.rw / t) * dv->num_sms, rounds = (nq + per_round - 1) / per_round;
+            const int64_t cost = rounds * (std::min(P.R, (groups + t - 1) / t * REF_CH) + 2);
+            if (cost < best) { best = cost; P.rteam = t; }
+        }
         P.rsm = cb + per * P.rw;
         auto kern = refine_kernel_for(P.rboth, dv->d, dv->bM > 1);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_PER_BLOCK) != cudaSuccess) {

@@ -1424,8 +1424,11 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     if (c1 + smem_per_warp > MAX_SMEM_PER_BLOCK) return cudaErrorInvalidConfiguration;
     int wpc = (int)std::min<size_t>(walk_threads(D1, FQ) / 32, (MAX_SMEM_PER_BLOCK - c1) / smem_per_warp);
     if (want > 0) wpc = std::min(wpc, want);
-    // a batch that does not fill the GPU spreads over all SMs
-    wpc = (int)std::min<int64_t>(wpc, std::max<int64_t>(1, (wa.nq + num_sms - 1) / num_sms));
+    // a batch that does not fill the GPU spreads over all SMs, evenly: one CTA on each (777 queries
+    // run as 152 CTAs of 6 warps, and not as 130)
+    const int64_t even = std::max<int64_t>(1, (wa.nq + num_sms - 1) / num_sms);
+    const bool small = even < wpc;
+    wpc = (int)std::min<int64_t>(wpc, even);
     size_t smem = c1 + smem_per_warp * wpc;
     // the attribute is an upper bound: set to the maximum, so plans made in any order (the
     // server plans at submission and launches later) all remain launchable
@@ -1436,7 +1439,7 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, wpc * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    int64_t need = (wa.nq + wpc - 1) / wpc;
+    const int64_t need = small ? std::min<int64_t>(wa.nq, num_sms) : (wa.nq + wpc - 1) / wpc;
     *grid_out = (int)std::min<int64_t>(need, (int64_t)per_sm * num_sms);
     *wpc_out = wpc;
     *smem_out = smem;
