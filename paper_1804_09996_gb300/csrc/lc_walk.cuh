@@ -132,10 +132,37 @@ struct WalkArgs {
     // null: position i is query i)
     int mode;
     const int32_t *order;
+    // ordered search with a re-rank: the queries walked so far, in the order they end (done_list
+    // [nq], -1 where none yet; done_tail entries taken), for the re-rank that starts meanwhile
+    int32_t *done_list, *done_tail;
     const __half *tab;     // table form: the queries' ADC tables [nq][256][M1] (FP16)
     int32_t *seed, *seed_up;
     float *seed_d;
 };
+
+// Programmatic dependent launch: the kernels of a search let the next one start as soon as SMs are
+// free (pdl_launch), and wait for the previous one to have ended (pdl_wait) once their codebooks
+// are in shared memory, before they touch anything it writes.  Each lets the next one start only
+// after its own wait, so a kernel that runs has everything of the kernels before the one ahead of it.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launches kern on st; pdl: it may start before the kernel queued ahead of it has ended.
+template <typename... P, typename... A>
+static cudaError_t launch(void (*kern)(P...), int64_t grid, int block, size_t smem, cudaStream_t st, bool pdl, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 constexpr int MAX_WALK_WARPS = 20;       // warps (queries in flight) per CTA
 // threads per CTA an instantiation is compiled for: the full-decode walk and the uneven splits
@@ -1011,6 +1038,10 @@ __device__ __forceinline__ void load_codebooks(const WalkArgs &a, unsigned char 
     }
     copy_wait();
     __syncthreads();
+    pdl_wait();
+    // only now may the next kernel start: what it reads without waiting for this one (the re-rank:
+    // the list of ended walks, reset by the queue sort) has to be there
+    pdl_launch();
 }
 
 // TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
@@ -1273,6 +1304,11 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             if (failed) atomicOr(a.status, 1);
         }
         __syncwarp();
+        if (a.done_list && lane == 0) {
+            __threadfence();                             // the shortlist (every lane's part) before the entry
+            asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.done_list + atomicAdd(a.done_tail, 1)), "r"((int32_t)q)
+                         : "memory");
+        }
     }
 }
 
@@ -1408,10 +1444,9 @@ struct WalkShape {
 };
 
 template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
-static cudaError_t run_descent(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st)
+static cudaError_t run_descent(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    descent_kernel<M1, D1, CT, FQ, TAB><<<grid, wpc * 32, smem, st>>>(wa);
-    return cudaGetLastError();
+    return launch(descent_kernel<M1, D1, CT, FQ, TAB>, grid, wpc * 32, smem, st, pdl, wa);
 }
 
 // Warps per CTA: as many as fit next to the codebook (at most MAX_WALK_WARPS, and at most
@@ -1447,10 +1482,9 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
 }
 
 template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
-static cudaError_t run_walk(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st)
+static cudaError_t run_walk(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    walk_kernel<M1, D1, CT, FQ, TAB, BATCH><<<grid, wpc * 32, smem, st>>>(wa);
-    return cudaGetLastError();
+    return launch(walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, grid, wpc * 32, smem, st, pdl, wa);
 }
 
 // Runs f(WalkShape<M1, D1, FQ>) for the instantiation of a sub-space width variant, M1 and the
@@ -1487,12 +1521,12 @@ static auto by_shape(int variant, int M1, bool fq, F &&f) -> decltype(f(WalkShap
     cudaError_t walk_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms, int want,    \
                                    int *wpc, int *grid, size_t *smem);                                                      \
     cudaError_t walk_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,           \
-                                cudaStream_t st);                                                                           \
+                                cudaStream_t st, bool pdl);                                                                 \
     const void *walk_fn_##NAME(int variant, int M1, bool fq, bool batch);                                                   \
     cudaError_t descent_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,       \
                                       size_t *smem);                                                                        \
     cudaError_t descent_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,        \
-                                   cudaStream_t st);
+                                   cudaStream_t st, bool pdl);
 WALK_ENTRIES(f32)
 WALK_ENTRIES(f16)
 WALK_ENTRIES(tab)
@@ -1506,9 +1540,10 @@ inline cudaError_t walk_config(WalkForm f, int variant, int M1, bool fq, const W
                                                                                               sms, want, wpc, grid, smem);
 }
 inline cudaError_t walk_run(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                            cudaStream_t st)
+                            cudaStream_t st, bool pdl)
 {
-    return (f == WALK_F32 ? walk_run_f32 : f == WALK_F16 ? walk_run_f16 : walk_run_tab)(variant, M1, fq, wa, smem, wpc, grid, st);
+    return (f == WALK_F32 ? walk_run_f32 : f == WALK_F16 ? walk_run_f16 : walk_run_tab)(variant, M1, fq, wa, smem, wpc, grid, st,
+                                                                                        pdl);
 }
 inline const void *walk_fn(WalkForm f, int variant, int M1, bool fq, bool batch)
 {
@@ -1521,10 +1556,10 @@ inline cudaError_t descent_config(WalkForm f, int variant, int M1, bool fq, cons
                                                                                                        sms, wpc, grid, smem);
 }
 inline cudaError_t descent_run(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                               cudaStream_t st)
+                               cudaStream_t st, bool pdl)
 {
     return (f == WALK_F32 ? descent_run_f32 : f == WALK_F16 ? descent_run_f16 : descent_run_tab)(variant, M1, fq, wa, smem, wpc,
-                                                                                              grid, st);
+                                                                                              grid, st, pdl);
 }
 
 }  // namespace lc

@@ -15,12 +15,12 @@ cudaError_t walk_config_f16(int variant, int M1, bool fq, const WalkArgs &wa, si
 }
 
 cudaError_t walk_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                         cudaStream_t st)
+                         cudaStream_t st, bool pdl)
 {
     return by_shape<__half>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? run_walk<T::M1, T::D1, __half, T::FQ, false, true>(wa, smem, wpc, grid, st)
-                           : run_walk<T::M1, T::D1, __half, T::FQ, false, false>(wa, smem, wpc, grid, st);
+        return wa.beam > 1 ? run_walk<T::M1, T::D1, __half, T::FQ, false, true>(wa, smem, wpc, grid, st, pdl)
+                           : run_walk<T::M1, T::D1, __half, T::FQ, false, false>(wa, smem, wpc, grid, st, pdl);
     });
 }
 
@@ -47,11 +47,11 @@ cudaError_t descent_config_f16(int variant, int M1, bool fq, const WalkArgs &wa,
 }
 
 cudaError_t descent_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                            cudaStream_t st)
+                            cudaStream_t st, bool pdl)
 {
     return by_shape<__half>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return run_descent<T::M1, T::D1, __half, T::FQ>(wa, smem, wpc, grid, st);
+        return run_descent<T::M1, T::D1, __half, T::FQ>(wa, smem, wpc, grid, st, pdl);
     });
 }
 
@@ -63,10 +63,10 @@ cudaError_t walk_config_tab(int, int, bool, const WalkArgs &wa, size_t per_warp,
                        : launch_walk<32, 3, __half, false, true, false>(wa, per_warp, sms, want, wpc, grid, smem);
 }
 
-cudaError_t walk_run_tab(int, int, bool, const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st)
+cudaError_t walk_run_tab(int, int, bool, const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    return wa.beam > 1 ? run_walk<32, 3, __half, false, true, true>(wa, smem, wpc, grid, st)
-                       : run_walk<32, 3, __half, false, true, false>(wa, smem, wpc, grid, st);
+    return wa.beam > 1 ? run_walk<32, 3, __half, false, true, true>(wa, smem, wpc, grid, st, pdl)
+                       : run_walk<32, 3, __half, false, true, false>(wa, smem, wpc, grid, st, pdl);
 }
 
 const void *walk_fn_tab(int, int, bool, bool batch)
@@ -80,9 +80,9 @@ cudaError_t descent_config_tab(int, int, bool, const WalkArgs &wa, int sms, int 
     return launch_descent<32, 3, __half, false, true>(wa, sms, wpc, grid, smem);
 }
 
-cudaError_t descent_run_tab(int, int, bool, const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st)
+cudaError_t descent_run_tab(int, int, bool, const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    return run_descent<32, 3, __half, false, true>(wa, smem, wpc, grid, st);
+    return run_descent<32, 3, __half, false, true>(wa, smem, wpc, grid, st, pdl);
 }
 
 }  // namespace lc

@@ -15,12 +15,12 @@ cudaError_t walk_config_f32(int variant, int M1, bool fq, const WalkArgs &wa, si
 }
 
 cudaError_t walk_run_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                         cudaStream_t st)
+                         cudaStream_t st, bool pdl)
 {
     return by_shape<float>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? run_walk<T::M1, T::D1, float, T::FQ, false, true>(wa, smem, wpc, grid, st)
-                           : run_walk<T::M1, T::D1, float, T::FQ, false, false>(wa, smem, wpc, grid, st);
+        return wa.beam > 1 ? run_walk<T::M1, T::D1, float, T::FQ, false, true>(wa, smem, wpc, grid, st, pdl)
+                           : run_walk<T::M1, T::D1, float, T::FQ, false, false>(wa, smem, wpc, grid, st, pdl);
     });
 }
 
@@ -47,11 +47,11 @@ cudaError_t descent_config_f32(int variant, int M1, bool fq, const WalkArgs &wa,
 }
 
 cudaError_t descent_run_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,
-                            cudaStream_t st)
+                            cudaStream_t st, bool pdl)
 {
     return by_shape<float>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return run_descent<T::M1, T::D1, float, T::FQ>(wa, smem, wpc, grid, st);
+        return run_descent<T::M1, T::D1, float, T::FQ>(wa, smem, wpc, grid, st, pdl);
     });
 }
 
