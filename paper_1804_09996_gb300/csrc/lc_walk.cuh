@@ -837,77 +837,102 @@ static __device__ __noinline__ bool overflow_insert(int32_t e, int32_t *stash, i
     return table_insert(e, spill, spill_log, 3);
 }
 
-// Tests and inserts the adjacency rows of NR nodes (ev[u]: this lane's entry of row u, -1: none);
-// appends the ids seen for the first time to slot[ns...] and returns their number.  The caller
-// has checked the limits for all rows.  Insertion without atomics (one warp owns the table, and a
-// compare-and-swap on random shared addresses takes 180 cycles alone and 1,024 with 16 warps per
-// SM): in each round the lanes that want to insert write their code to their bucket's owner byte
-// (shared by buckets OWNERS apart), and the one that is read back stores its entry; the others look again, so an id in two rows
-// (or twice in one) is fresh once.  Two rounds are typical (four rows bring about 36 new ids,
-// some of them twice, to 256 buckets).
-template <bool TAG, int NR>
-__device__ __forceinline__ int visit_rows(Visited &V, const VisitTab &vt, int spill_log, const int32_t (&ev)[NR],
+// Tests and inserts one id per lane (e < 0: none) into the visited set; appends those that were not
+// there to slot[ns...] and returns their number.  Insertion without atomics (one warp owns the
+// table, and a compare-and-swap on random shared addresses takes 180 cycles alone and 1,024 with 16
+// warps per SM): in each round the lanes that want to insert write their lane to their bucket's
+// owner byte (shared by buckets OWNERS apart), and the one that is read back stores its entry; the
+// others look again, so an id that two lanes hold is fresh once.
+template <bool TAG>
+__device__ __forceinline__ int visit_ids(Visited &V, const VisitTab &vt, int spill_log, int32_t e, int32_t *slot, int ns,
+                                         int lane)
+{
+    const bool closed = !TAG && V.spilled;
+    int32_t todo = e;
+    bool fresh = false, over = false;
+    do {
+        uint32_t at, own = 0, nw;
+        const int r = bucket_probe<TAG>(vt, V.tab_s, todo, closed, &at, &own, &nw);
+        over |= r == VISIT_OVERFLOW;
+        if (r != VISIT_INSERT) todo = -1;
+        own = V.own_s + (own & (OWNERS - 1));
+        if (todo >= 0) asm volatile("st.shared.u8 [%0], %1;" ::"r"(own), "r"(lane) : "memory");
+        __syncwarp();
+        uint32_t c = 0xff;
+        if (todo >= 0) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(c) : "r"(own) : "memory");
+        __syncwarp();
+        if (c == (uint32_t)lane) {
+            bucket_store<TAG>(at, nw);
+            fresh = true;
+            todo = -1;
+        }
+        __syncwarp();
+    } while (__any_sync(FULL, todo >= 0));
+    const unsigned ov = __ballot_sync(FULL, over);
+    if (ov) {
+        if (TAG && !V.stash_full && V.ocount + __popc(ov) > shared_visited_cap(1 << vt.stash_log)) {
+            V.stash_full = true;
+            clear_spill(V.spill, spill_log, lane);
+        }
+        if (over) fresh = overflow_insert(e, V.stash, TAG ? vt.stash_log : -1, V.stash_full, V.spill, spill_log);
+        if (!V.stash_full) V.ocount += __popc(ov);       // (at most)
+        __syncwarp();
+    }
+    const unsigned m = __ballot_sync(FULL, fresh);
+    if (fresh) slot[ns + __popc(m & ((1u << lane) - 1))] = e;
+    return __popc(m);
+}
+
+// The same for the adjacency rows of cnt <= 4 nodes (ev[u]: this lane's entry of row u, -1: none);
+// the caller has checked the limits for all rows.  The four rows go through one round together;
+// the few ids that lose their bucket in it (four rows bring about 36 new ids, some of them twice,
+// to 256 buckets) or find it full are gathered behind the fresh ones, at the end of the rows' part
+// of slot[], and go through visit_ids: a second round of all four rows would be mostly idle
+// (10k queries, beam 4: 650 -> 610 us).
+template <bool TAG>
+__device__ __forceinline__ int visit_rows(Visited &V, const VisitTab &vt, int spill_log, const int32_t (&ev)[4], int cnt,
                                           int32_t *slot, int ns, int lane)
 {
     const bool closed = !TAG && V.spilled;
-    unsigned todo = 0, fresh = 0, over = 0;              // bit u: row u's entry
-#pragma unroll
-    for (int u = 0; u < NR; u++) todo |= (unsigned)(ev[u] >= 0) << u;
-    do {
-        uint32_t at[NR], own[NR] = {}, nw[NR];
-#pragma unroll
-        for (int u = 0; u < NR; u++) {
-            const int r = bucket_probe<TAG>(vt, V.tab_s, (todo >> u) & 1 ? ev[u] : -1, closed, &at[u], &own[u], &nw[u]);
-            over |= (unsigned)(r == VISIT_OVERFLOW) << u;
-            if (r != VISIT_INSERT) todo &= ~(1u << u);
-            own[u] = V.own_s + (own[u] & (OWNERS - 1));
-        }
-#pragma unroll
-        for (int u = 0; u < NR; u++)
-            if ((todo >> u) & 1)
-                asm volatile("st.shared.u8 [%0], %1;" ::"r"(own[u]), "r"(lane | (u << 5)) : "memory");
-        __syncwarp();
-        unsigned won = 0;
-#pragma unroll
-        for (int u = 0; u < NR; u++) {
-            uint32_t c = 0xff;
-            if ((todo >> u) & 1) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(c) : "r"(own[u]) : "memory");
-            won |= (unsigned)(c == (uint32_t)(lane | (u << 5))) << u;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < NR; u++)
-            if ((won >> u) & 1) bucket_store<TAG>(at[u], nw[u]);
-        fresh |= won;
-        todo &= ~won;
-        __syncwarp();
-    } while (__any_sync(FULL, todo != 0));
-    if (__any_sync(FULL, over != 0)) {
-#pragma unroll 1
-        for (int u = 0; u < NR; u++) {
-            const unsigned ov = __ballot_sync(FULL, (over >> u) & 1);
-            if (!ov) continue;
-            int32_t e = ev[0];
-#pragma unroll
-            for (int i = 1; i < NR; i++) e = u == i ? ev[i] : e;
-            if (TAG && !V.stash_full && V.ocount + __popc(ov) > shared_visited_cap(1 << vt.stash_log)) {
-                V.stash_full = true;
-                clear_spill(V.spill, spill_log, lane);
-            }
-            if ((over >> u) & 1)
-                fresh |= (unsigned)overflow_insert(e, V.stash, TAG ? vt.stash_log : -1, V.stash_full, V.spill, spill_log) << u;
-            if (!V.stash_full) V.ocount += __popc(ov);   // (at most)
-            __syncwarp();
-        }
-    }
     const unsigned lt_mask = (1u << lane) - 1;
-    int n = ns;
+    uint32_t at[4], own[4] = {}, nw[4];
+    int r[4];
 #pragma unroll
-    for (int u = 0; u < NR; u++) {
-        const bool f = (fresh >> u) & 1;
-        const unsigned m = __ballot_sync(FULL, f);
-        if (f) slot[n + __popc(m & lt_mask)] = ev[u];
+    for (int u = 0; u < 4; u++) {
+        r[u] = bucket_probe<TAG>(vt, V.tab_s, ev[u], closed, &at[u], &own[u], &nw[u]);
+        own[u] = V.own_s + (own[u] & (OWNERS - 1));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++)
+        if (r[u] == VISIT_INSERT) asm volatile("st.shared.u8 [%0], %1;" ::"r"(own[u]), "r"(lane | (u << 5)) : "memory");
+    __syncwarp();
+    bool won[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        uint32_t c = 0xff;
+        if (r[u] == VISIT_INSERT) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(c) : "r"(own[u]) : "memory");
+        won[u] = c == (uint32_t)(lane | (u << 5));
+    }
+    __syncwarp();
+    int n = ns, end = ns + 32 * cnt;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+        const unsigned m = __ballot_sync(FULL, won[u]), l = __ballot_sync(FULL, r[u] != VISIT_SEEN && !won[u]);
+        if (won[u]) {
+            bucket_store<TAG>(at[u], nw[u]);
+            slot[n + __popc(m & lt_mask)] = ev[u];
+        } else if (r[u] != VISIT_SEEN) {
+            slot[end - 1 - __popc(l & lt_mask)] = ev[u];
+        }
         n += __popc(m);
+        end -= __popc(l);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int c = end; c < ns + 32 * cnt; c += 32) {      // (n <= end throughout: each id is listed once)
+        const int32_t e = c + lane < ns + 32 * cnt ? slot[c + lane] : -1;
+        __syncwarp();
+        n += visit_ids<TAG>(V, vt, spill_log, e, slot, n, lane);
     }
     return n - ns;
 }
@@ -929,7 +954,7 @@ static __device__ __noinline__ int visit_rows_ids(uint32_t tab, uint32_t owners,
     int32_t ev[4];
 #pragma unroll
     for (int u = 0; u < 4; u++) ev[u] = u < cnt ? __ldg(adj0 + (int64_t)sel[u] * DEG + lane) : -1;
-    return visit_rows<false, 4>(V, vt, spill_log, ev, slot, ns, lane);
+    return visit_rows<false>(V, vt, spill_log, ev, cnt, slot, ns, lane);
 }
 
 // Members of the sorted list W (wn keys) below k: four-way search, three reads a step in flight
@@ -1205,13 +1230,12 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                         nf = visit_rows_ids(V.tab_s, V.own_s, a.vt.bb, V.spill, a.spill_log, V.spilled, a.adj0, sel + r0,
                                             cnt, slot, ns, lane);
                     } else if constexpr (!BATCH) {
-                        const int32_t ev[1] = {__ldg(a.adj0 + (int64_t)sel[r0] * DEG + lane)};
-                        nf = visit_rows<true, 1>(V, a.vt, a.spill_log, ev, slot, ns, lane);
+                        nf = visit_ids<true>(V, a.vt, a.spill_log, __ldg(a.adj0 + (int64_t)sel[r0] * DEG + lane), slot, ns, lane);
                     } else {
                         int32_t ev[4];
 #pragma unroll
                         for (int u = 0; u < 4; u++) ev[u] = u < cnt ? __ldg(a.adj0 + (int64_t)sel[r0 + u] * DEG + lane) : -1;
-                        nf = visit_rows<true, 4>(V, a.vt, a.spill_log, ev, slot, ns, lane);
+                        nf = visit_rows<true>(V, a.vt, a.spill_log, ev, cnt, slot, ns, lane);
                     }
                     ns += nf;
                     n_dist += nf;
