@@ -115,7 +115,7 @@ struct SearchPlan {
     bool refine = false;
     bool half = false;                   // FP16 level-1 codebook in the walk
     bool full = false;                   // the walk scores the full two-level decode
-    int wpc = 0, grid = 0;               // walk: warps per CTA, CTAs
+    int wpc = 0, grid = 0, team = 1;     // walk: queries per CTA, CTAs, warps per query
     size_t per_warp = 0, smem = 0;
     int rw = 0, rgrid = 0, rteam = 1;    // refine: warps per CTA, CTAs, warps per query
     size_t rsm = 0;

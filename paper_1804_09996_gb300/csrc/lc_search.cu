@@ -761,6 +761,7 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     } else {
         P.tab_elems = P.tab ? (size_t)nq * 256 * TAB_M1 : 0;
         wa.beam = P.beam;
+        P.team = wa.team = P.tab || sp->warps ? 1 : walk_team(nq, dv->num_sms, dv->M1);
         ce = walk_config(P.form(), P.variant, dv->M1, P.full, wa, P.per_warp, dv->num_sms, sp->warps, &P.wpc, &P.grid, &P.smem);
     }
     if (ce == cudaErrorInvalidConfiguration) {
@@ -852,6 +853,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     wa.efp = P.efp; wa.efcap = (int)align_up(P.efp, 32);
     wa.R = P.R; wa.refine = P.refine ? 1 : 0;
     wa.beam = P.beam;
+    wa.team = P.team;
     wa.tcap = P.tcap;
     wa.hash_log = P.hash_log;
     wa.spill_log = P.spill_log;
@@ -1494,7 +1496,7 @@ lc_status plan_create(lc_index *ix, int64_t nq_max, const lc_search_params *sp, 
     // find the two kernel nodes whose batch size a smaller call updates
     // (the rotation and, in the table form, the table launch keep the largest batch: their
     // extra rows are computed and not read)
-    const void *wf = walk_fn(P.form(), P.variant, dv->M1, P.full, P.beam > 1);
+    const void *wf = walk_fn(P.form(), P.variant, dv->M1, P.full, P.beam > 1, P.team > 1);
     const void *rf = P.refine ? (const void *)refine_kernel_for(P.rboth, d, dv->bM > 1) : nullptr;
     size_t nn = 0;
     cudaGraphGetNodes(pl->graph, nullptr, &nn);

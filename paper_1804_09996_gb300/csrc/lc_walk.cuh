@@ -105,6 +105,7 @@ struct WalkArgs {
     int R;            // shortlist length (refine) or k (no refinement)
     int refine;
     int beam;         // expansions per step (1: the plain walk)
+    int team;         // > 1: warps per query (small batches)
     int tcap;         // > 0: stop once that many level-0 distances were computed
     int hash_log;     // visited-set limits: 2^hash_log entries (see VisitTab) ...
     int spill_log;    // ... and a global table of 2^spill_log entries per query in flight
@@ -177,7 +178,7 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 // Shared memory of the walk kernel: the level-1 codebook C1 [256][d] once per CTA, then one
 // region per warp.
 struct WalkSmem {
-    size_t yq, stage, wkey, cand, sel, slot, hash, total;
+    size_t yq, stage, wkey, cand, sel, ctl, slot, hash, total;
 };
 
 // Layout of the walk's level-1 codebook in shared memory, chosen so that a lane's sub-space
@@ -223,13 +224,11 @@ inline int walk_variant(int M1, int d)
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__half x) { return __half2float(x); }
 
-// Nodes whose code rows are staged together: two chunks of 32 where a step can have that many
-// fresh nodes (beam > 1) and a row is at most 32 bytes, so that most steps wait for global memory
-// once; one chunk otherwise (a second one would cost walks in flight).
-__host__ __device__ constexpr int stage_rows(int row_bytes, int beam, int tag)
-{
-    return tag && beam > 1 && row_bytes <= 32 ? 64 : 32;
-}
+// Nodes whose code rows are staged together.  (64 where a step of the batched walk can have that
+// many, so that it waits for global memory once, cost walks in flight: 2,318 against 2,195 us at
+// efSearch 128 on 3M vectors.)
+constexpr int STAGE_ROWS = 32;
+
 // own_rot: the walk rotates the query itself (y' in shared memory); otherwise y' is read from
 // the rotation kernel's output.
 __host__ __device__ inline WalkSmem walk_smem(int M1, int d, int efcap, const VisitTab &vt, int beam, bool own_rot,
@@ -238,10 +237,11 @@ __host__ __device__ inline WalkSmem walk_smem(int M1, int d, int efcap, const Vi
     WalkSmem s;
     size_t o = 0;
     s.yq = o;        o += own_rot ? align_up((size_t)d * 4, 16) : 0;
-    s.stage = o;     o += (size_t)stage_rows(M1 + m2p, beam, vt.tag) * (M1 + m2p);   // level-1 rows, then residual rows
+    s.stage = o;     o += (size_t)STAGE_ROWS * (M1 + m2p);   // level-1 rows, then residual rows
     s.wkey = o;      o += (size_t)efcap * 8;
     s.cand = o;      o += (size_t)32 * beam * 8 + 32;                          // candidates of a step, padded
     s.sel = o;       o += 32;                                                // nodes expanded in a step (at most 8)
+    s.ctl = o;       o += 16;                                                // team: query, nodes to score
     s.slot = o;      o += (size_t)32 * beam * 4;
     s.hash = o;      o += visit_bytes(vt);
     s.total = align_up(o, 128);
@@ -615,24 +615,19 @@ __device__ __forceinline__ void copy_async(void *dst, const void *src, size_t by
         copy16(static_cast<char *>(dst) + i, static_cast<const char *>(src) + i);
 }
 
-// Code rows of the n nodes in slot[0..n) (n <= rows) into the staging area: the level-1 rows,
-// then, for the full walk, the residual rows behind all `rows` of them.
+// Code rows of the n <= STAGE_ROWS nodes in slot[0..n) into the staging area: the level-1 rows,
+// then, for the full walk, the residual rows behind all of them.
 template <int M1, bool FQ>
-__device__ __forceinline__ void stage_codes(uint8_t *stage, int rows, const uint8_t *codes1, const uint8_t *codes2b, int M2P,
+__device__ __forceinline__ void stage_codes(uint8_t *stage, const uint8_t *codes1, const uint8_t *codes2b, int M2P,
                                             const int32_t *slot, int n, int lane)
 {
     __syncwarp();                                        // slot written, the staged rows read
+    if (lane < n) {
+        const int64_t v = slot[lane];
 #pragma unroll
-    for (int i0 = 0; i0 < 64; i0 += 32) {
-        if (i0 >= n) break;
-        const int i = i0 + lane;
-        if (i < n) {
-            const int64_t v = slot[i];
-#pragma unroll
-            for (int u = 0; u < M1 / 16; u++) copy16(stage + i * M1 + 16 * u, codes1 + v * M1 + 16 * u);
-            if constexpr (FQ)
-                for (int u = 0; u < M2P; u += 16) copy16(stage + rows * M1 + i * M2P + u, codes2b + v * M2P + u);
-        }
+        for (int u = 0; u < M1 / 16; u++) copy16(stage + lane * M1 + 16 * u, codes1 + v * M1 + 16 * u);
+        if constexpr (FQ)
+            for (int u = 0; u < M2P; u += 16) copy16(stage + STAGE_ROWS * M1 + lane * M2P + u, codes2b + v * M2P + u);
     }
     copy_wait();
     __syncwarp();
@@ -1071,15 +1066,50 @@ __device__ __forceinline__ void load_codebooks(const WalkArgs &a, unsigned char 
 
 // TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
 // [256][M1] (FP16, built by table_kernel) in shared memory and scores nodes by table lookups.
+// A team's share of scoring the n nodes in slot[0..n): blocks of slot_block nodes in turn, each
+// staged and scored by one warp, totals into dist[0..n).  Block b takes the rows from b * SB mod STAGE_ROWS
+// of the staging area; the team's size divides their number, so the rows of a warp are its own.
+template <int M1, int D1, typename CT, bool FQ>
+__device__ __forceinline__ void score_team(const CT *C1s, uint8_t *stage, const uint8_t *codes1, const uint8_t *codes2b, int M2P,
+                                            const int32_t *slot, int n, int d, const LaneGeo<M1, D1> &g, int lane,
+                                           int tw, int W, const CT *C2, float *dist)
+{
+    constexpr int SB = slot_block(M1), P1 = M1 / 16;
+    const int s3 = slot_of_lane(lane, 3), node = M1 == 16 ? 2 * s3 + (lane >> 4) : s3;
+#pragma unroll 1
+    for (int b = tw; b * SB < n; b += W) {
+        const int row0 = (b * SB) % STAGE_ROWS, r = lane / P1;
+        uint8_t *st = stage + row0 * M1, *st2 = stage + STAGE_ROWS * M1 + row0 * M2P;
+        if (r < SB && b * SB + r < n)
+            copy16(st + lane * 16, codes1 + (int64_t)slot[b * SB + r] * M1 + (lane % P1) * 16);
+        if constexpr (FQ)
+            if (lane < SB && b * SB + lane < n)
+                for (int u = 0; u < M2P; u += 16) copy16(st2 + lane * M2P + u, codes2b + (int64_t)slot[b * SB + lane] * M2P + u);
+        copy_wait();
+        __syncwarp();
+        float v[8];
+        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, false, false>(C1s, st, st2, d, g, lane, C2, M2P, v);
+        else block_terms<M1, D1, CT, FQ, false, true>(C1s, st, st2, d, g, lane, C2, M2P, v);
+        const float t = reduce_block<M1>(v);
+        if (lane_block<M1>(lane) == 0 && b * SB + node < n) dist[b * SB + node] = t;
+        __syncwarp();
+    }
+}
+
+// TEAM: a.team warps per query, for batches that leave most of an SM idle: the first walks, the
+// others stage and score their share of each step's nodes (between two named barriers).  It
+// shortens a step, which bounds a small batch (16 queries 247 -> 227 us, one 94 -> 84), and wastes
+// issue slots in a large one.
 // BATCH: beam > 1.  The plain walk is an instantiation of its own: it visits one row and merges at
 // most 32 candidates a step, and the step's code has to stay small (the instruction cache bounds
 // it: with the code for four rows beside its own the plain walk of 10k queries took 908 and not
 // 853 us).
-template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH, bool TEAM>
 __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, team = TEAM ? a.team : 1;
+    const int warp = TEAM ? (threadIdx.x >> 5) / team : threadIdx.x >> 5, tw = TEAM ? (threadIdx.x >> 5) % team : 0;
     const int d = a.d;
     // the level-1 codebook, shared by every warp of the CTA
     CT *C1s = reinterpret_cast<CT *>(smem_raw);
@@ -1095,21 +1125,28 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
     uint64_t *cand = reinterpret_cast<uint64_t *>(base + L.cand);
     int32_t *sel = reinterpret_cast<int32_t *>(base + L.sel);
     int32_t *slot = reinterpret_cast<int32_t *>(base + L.slot);
-    const int SR = BATCH ? stage_rows(M1 + (FQ ? a.M2P : 0), a.beam, a.vt.tag) : 32;
-    const int64_t gwarp = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+    volatile int32_t *ctl = reinterpret_cast<int32_t *>(base + L.ctl);
+    float *dist = reinterpret_cast<float *>(cand) + 32 * a.beam;             // (read before candidates reach it)
+    auto team_bar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + warp), "r"(team * 32) : "memory"); };
+    const int64_t gwarp = (int64_t)blockIdx.x * ((blockDim.x >> 5) / team) + warp;
     Visited V;
     V.tab = base + L.hash;
     V.tab_s = (uint32_t)__cvta_generic_to_shared(V.tab);
     V.stash = reinterpret_cast<int32_t *>(base + L.hash + a.vt.bytes);
     V.own_s = (uint32_t)__cvta_generic_to_shared(base + L.stage);
     const int H = 1 << a.hash_log;
-    const int my_slot = chunk_slot<M1>(lane);
+    const int my_slot = TEAM ? lane : chunk_slot<M1>(lane);
     const unsigned lt_mask = (1u << lane) - 1;
 
     for (;;) {
         int64_t qi = 0;
-        if (lane == 0) qi = atomicAdd(a.counter, 1ull);
+        if (lane == 0 && tw == 0) qi = atomicAdd(a.counter, 1ull);
         qi = __shfl_sync(FULL, qi, 0);
+        if constexpr (TEAM) {
+            if (tw == 0 && lane == 0) ctl[0] = (int32_t)min(qi, (int64_t)0x7fffffff);
+            team_bar();
+            qi = ctl[0];
+        }
         if (qi >= a.nq) break;
         const int64_t q = a.order ? (int64_t)__ldg(a.order + qi) : qi;
         V.spill = a.spill + ((a.spill_tables >= a.nq ? qi : gwarp) << a.spill_log);
@@ -1145,10 +1182,22 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
                 yq[t] = s;
             }
         }
-        V.clear(a.vt, lane);
+        if (tw == 0) V.clear(a.vt, lane);
         __syncwarp();
         LaneGeo<M1, D1> g;
         g.init(a.s1, yrot, FQ ? a.sub2 : nullptr, d, lane);
+        if constexpr (TEAM) {
+            if (tw > 0) {
+                for (;;) {
+                    team_bar();
+                    const int n = ctl[1];
+                    if (n == 0) break;                   // the walk has ended
+                    score_team<M1, D1, CT, FQ>(C1s, stage, a.codes1, a.codes2b, a.M2P, slot, n, d, g, lane, tw, team, C2, dist);
+                    team_bar();
+                }
+                continue;
+            }
+        }
         // One loop runs the greedy descent of the upper levels (Section 2) and then the level-0
         // best-first search.  Each iteration gathers the nodes to score in slot[] and scores
         // them at a single call site, so the kernel holds one copy of the scoring code.
@@ -1253,13 +1302,19 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             uint32_t bd = ~0u, bi = ~0u;
             const uint64_t wmax = phase == 2 && wn == efp ? W[wn - 1] : ~0ull;
             int nc = 0;
+            if constexpr (TEAM) {
+                if (lane == 0) ctl[1] = ns;
+                team_bar();
+                score_team<M1, D1, CT, FQ>(C1s, stage, a.codes1, a.codes2b, a.M2P, slot, ns, d, g, lane, 0, team, C2, dist);
+                team_bar();
+            }
 #pragma unroll 1
             for (int ch = 0; ch < ns; ch += 32) {          // (once unless BATCH)
-                const int at = BATCH ? ch % SR : 0;                  // place in the staging area
-                if (at == 0) stage_codes<M1, FQ>(stage, SR, a.codes1, a.codes2b, a.M2P, slot + ch, min(SR, ns - ch), lane);
                 const int nf = min(32, ns - ch);
-                const float de = score_staged<M1, D1, CT, FQ, TAB, BATCH && !FQ && (D1 > 0)>(C1s, stage + at * M1, stage + SR * M1 + at * a.M2P, nf, d, g,
-                                                                   lane, C2, a.M2P);
+                if (!TEAM) stage_codes<M1, FQ>(stage, a.codes1, a.codes2b, a.M2P, slot + ch, nf, lane);
+                float de;
+                if constexpr (TEAM) de = lane < nf ? dist[ch + lane] : 0.f;
+                else de = score_staged<M1, D1, CT, FQ, TAB, BATCH && !FQ && (D1 > 0)>(C1s, stage, stage + STAGE_ROWS * M1, nf, d, g, lane, C2, a.M2P);
                 const int32_t id = my_slot < nf ? slot[ch + my_slot] : -1;
                 if (phase < 2) {                         // at most 32 nodes here
                     warp_best(id >= 0 ? __float_as_uint(de) : ~0u, (uint32_t)id, &bd, &bi);
@@ -1303,6 +1358,10 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             }
         }
 
+        if constexpr (TEAM) {
+            if (lane == 0) ctl[1] = 0;
+            team_bar();
+        }
         // outputs
         if (a.refine) {
             if (!a.yq_in)
@@ -1402,7 +1461,7 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
             }
             uint32_t bd = ~0u, bi = ~0u;
             if (ns > 0) {
-                stage_codes<M1, FQ>(stage, 32, a.codes1, a.codes2b, a.M2P, slot, ns, lane);
+                stage_codes<M1, FQ>(stage, a.codes1, a.codes2b, a.M2P, slot, ns, lane);
                 const float de = score_staged<M1, D1, CT, FQ, TAB, !FQ && (D1 > 0)>(T1, stage, stage + 32 * M1, ns, d, g, lane, C2, a.M2P);
                 const int32_t id = my_slot < ns ? slot[my_slot] : -1;
                 warp_best(id >= 0 ? __float_as_uint(de) : ~0u, (uint32_t)id, &bd, &bi);
@@ -1430,6 +1489,14 @@ __global__ void __launch_bounds__(descent_threads(FQ)) descent_kernel(const Walk
 }
 
 constexpr size_t MAX_SMEM_PER_BLOCK = 227 * 1024;
+
+// Warps per query of a batch of nq: four while no SM has more than four queries (two for M1 = 16,
+// whose staging area holds two blocks), else one: with six queries an SM two warps each took 183
+// us where one took 179.
+inline int walk_team(int64_t nq, int sms, int M1)
+{
+    return nq > 4 * (int64_t)sms ? 1 : M1 == 16 ? 2 : 4;
+}
 
 // Launch shape of the descent: as many warps as fit next to the codebook, at most 32.
 template <int M1, int D1, typename CT, bool FQ, bool TAB = false>
@@ -1475,7 +1542,7 @@ static cudaError_t run_descent(const WalkArgs &wa, size_t smem, int wpc, int gri
 
 // Warps per CTA: as many as fit next to the codebook (at most MAX_WALK_WARPS, and at most
 // want if want > 0).
-template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH, bool TEAM>
 static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num_sms, int want, int *wpc_out,
                                int *grid_out, size_t *smem_out)
 {
@@ -1483,6 +1550,7 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     if (c1 + smem_per_warp > MAX_SMEM_PER_BLOCK) return cudaErrorInvalidConfiguration;
     int wpc = (int)std::min<size_t>(walk_threads(D1, FQ) / 32, (MAX_SMEM_PER_BLOCK - c1) / smem_per_warp);
     if (want > 0) wpc = std::min(wpc, want);
+    if (TEAM) wpc = std::min(wpc, std::min(15, walk_threads(D1, FQ) / 32 / wa.team));      // (a named barrier each)
     // a batch that does not fill the GPU spreads over all SMs, evenly: one CTA on each (777 queries
     // run as 152 CTAs of 6 warps, and not as 130)
     const int64_t even = std::max<int64_t>(1, (wa.nq + num_sms - 1) / num_sms);
@@ -1491,11 +1559,12 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     size_t smem = c1 + smem_per_warp * wpc;
     // the attribute is an upper bound: set to the maximum, so plans made in any order (the
     // server plans at submission and launches later) all remain launchable
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(walk_kernel<M1, D1, CT, FQ, TAB, BATCH, TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)MAX_SMEM_PER_BLOCK);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, wpc * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<M1, D1, CT, FQ, TAB, BATCH, TEAM>,
+                                                      wpc * (TEAM ? wa.team : 1) * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int64_t need = small ? std::min<int64_t>(wa.nq, num_sms) : (wa.nq + wpc - 1) / wpc;
@@ -1505,10 +1574,10 @@ static cudaError_t launch_walk(const WalkArgs &wa, size_t smem_per_warp, int num
     return cudaSuccess;
 }
 
-template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH>
+template <int M1, int D1, typename CT, bool FQ, bool TAB, bool BATCH, bool TEAM>
 static cudaError_t run_walk(const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    return launch(walk_kernel<M1, D1, CT, FQ, TAB, BATCH>, grid, wpc * 32, smem, st, pdl, wa);
+    return launch(walk_kernel<M1, D1, CT, FQ, TAB, BATCH, TEAM>, grid, wpc * (TEAM ? wa.team : 1) * 32, smem, st, pdl, wa);
 }
 
 // Runs f(WalkShape<M1, D1, FQ>) for the instantiation of a sub-space width variant, M1 and the
@@ -1540,13 +1609,14 @@ static auto by_shape(int variant, int M1, bool fq, F &&f) -> decltype(f(WalkShap
 
 // Launch shape, launch and kernel address of the walk, launch shape and launch of the descent, per
 // codebook element type (lc_walk_f32.cu, lc_walk_f16.cu) and for the table form (LC_LUT_TABLE;
-// M1 = 32 at d = 96).  Which walk instantiation also depends on wa.beam (walk_fn: batch).
+// M1 = 32 at d = 96).  Which walk instantiation also depends on wa.beam and wa.team (walk_fn:
+// batch, team).
 #define WALK_ENTRIES(NAME)                                                                                                  \
     cudaError_t walk_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t per_warp, int sms, int want,    \
                                    int *wpc, int *grid, size_t *smem);                                                      \
     cudaError_t walk_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,           \
                                 cudaStream_t st, bool pdl);                                                                 \
-    const void *walk_fn_##NAME(int variant, int M1, bool fq, bool batch);                                                   \
+    const void *walk_fn_##NAME(int variant, int M1, bool fq, bool batch, bool team);                                        \
     cudaError_t descent_config_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,       \
                                       size_t *smem);                                                                        \
     cudaError_t descent_run_##NAME(int variant, int M1, bool fq, const WalkArgs &wa, size_t smem, int wpc, int grid,        \
@@ -1569,9 +1639,9 @@ inline cudaError_t walk_run(WalkForm f, int variant, int M1, bool fq, const Walk
     return (f == WALK_F32 ? walk_run_f32 : f == WALK_F16 ? walk_run_f16 : walk_run_tab)(variant, M1, fq, wa, smem, wpc, grid, st,
                                                                                         pdl);
 }
-inline const void *walk_fn(WalkForm f, int variant, int M1, bool fq, bool batch)
+inline const void *walk_fn(WalkForm f, int variant, int M1, bool fq, bool batch, bool team)
 {
-    return (f == WALK_F32 ? walk_fn_f32 : f == WALK_F16 ? walk_fn_f16 : walk_fn_tab)(variant, M1, fq, batch);
+    return (f == WALK_F32 ? walk_fn_f32 : f == WALK_F16 ? walk_fn_f16 : walk_fn_tab)(variant, M1, fq, batch, team);
 }
 inline cudaError_t descent_config(WalkForm f, int variant, int M1, bool fq, const WalkArgs &wa, int sms, int *wpc, int *grid,
                                   size_t *smem)

@@ -9,8 +9,11 @@ cudaError_t walk_config_f16(int variant, int M1, bool fq, const WalkArgs &wa, si
 {
     return by_shape<__half>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? launch_walk<T::M1, T::D1, __half, T::FQ, false, true>(wa, per_warp, sms, want, wpc, grid, smem)
-                           : launch_walk<T::M1, T::D1, __half, T::FQ, false, false>(wa, per_warp, sms, want, wpc, grid, smem);
+        const auto fn = wa.team > 1 ? (wa.beam > 1 ? launch_walk<T::M1, T::D1, __half, T::FQ, false, true, true>
+                                                   : launch_walk<T::M1, T::D1, __half, T::FQ, false, false, true>)
+                                    : (wa.beam > 1 ? launch_walk<T::M1, T::D1, __half, T::FQ, false, true, false>
+                                                   : launch_walk<T::M1, T::D1, __half, T::FQ, false, false, false>);
+        return fn(wa, per_warp, sms, want, wpc, grid, smem);
     });
 }
 
@@ -19,19 +22,24 @@ cudaError_t walk_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, size_
 {
     return by_shape<__half>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? run_walk<T::M1, T::D1, __half, T::FQ, false, true>(wa, smem, wpc, grid, st, pdl)
-                           : run_walk<T::M1, T::D1, __half, T::FQ, false, false>(wa, smem, wpc, grid, st, pdl);
+        const auto fn = wa.team > 1 ? (wa.beam > 1 ? run_walk<T::M1, T::D1, __half, T::FQ, false, true, true>
+                                                   : run_walk<T::M1, T::D1, __half, T::FQ, false, false, true>)
+                                    : (wa.beam > 1 ? run_walk<T::M1, T::D1, __half, T::FQ, false, true, false>
+                                                   : run_walk<T::M1, T::D1, __half, T::FQ, false, false, false>);
+        return fn(wa, smem, wpc, grid, st, pdl);
     });
 }
 
 // The walk instantiation a plan launches (for finding its node in a captured graph).
-const void *walk_fn_f16(int variant, int M1, bool fq, bool batch)
+const void *walk_fn_f16(int variant, int M1, bool fq, bool batch, bool team)
 {
     const void *fn = nullptr;
     by_shape<__half>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        fn = batch ? (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, true>
-                   : (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, false>;
+        fn = team ? (batch ? (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, true, true>
+                           : (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, false, true>)
+                  : (batch ? (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, true, false>
+                           : (const void *)walk_kernel<T::M1, T::D1, __half, T::FQ, false, false, false>);
         return cudaSuccess;
     });
     return fn;
@@ -59,20 +67,20 @@ cudaError_t descent_run_f16(int variant, int M1, bool fq, const WalkArgs &wa, si
 cudaError_t walk_config_tab(int, int, bool, const WalkArgs &wa, size_t per_warp, int sms, int want, int *wpc, int *grid,
                             size_t *smem)
 {
-    return wa.beam > 1 ? launch_walk<32, 3, __half, false, true, true>(wa, per_warp, sms, want, wpc, grid, smem)
-                       : launch_walk<32, 3, __half, false, true, false>(wa, per_warp, sms, want, wpc, grid, smem);
+    return wa.beam > 1 ? launch_walk<32, 3, __half, false, true, true, false>(wa, per_warp, sms, want, wpc, grid, smem)
+                       : launch_walk<32, 3, __half, false, true, false, false>(wa, per_warp, sms, want, wpc, grid, smem);
 }
 
 cudaError_t walk_run_tab(int, int, bool, const WalkArgs &wa, size_t smem, int wpc, int grid, cudaStream_t st, bool pdl)
 {
-    return wa.beam > 1 ? run_walk<32, 3, __half, false, true, true>(wa, smem, wpc, grid, st, pdl)
-                       : run_walk<32, 3, __half, false, true, false>(wa, smem, wpc, grid, st, pdl);
+    return wa.beam > 1 ? run_walk<32, 3, __half, false, true, true, false>(wa, smem, wpc, grid, st, pdl)
+                       : run_walk<32, 3, __half, false, true, false, false>(wa, smem, wpc, grid, st, pdl);
 }
 
-const void *walk_fn_tab(int, int, bool, bool batch)
+const void *walk_fn_tab(int, int, bool, bool batch, bool)
 {
-    return batch ? (const void *)walk_kernel<32, 3, __half, false, true, true>
-                 : (const void *)walk_kernel<32, 3, __half, false, true, false>;
+    return batch ? (const void *)walk_kernel<32, 3, __half, false, true, true, false>
+                 : (const void *)walk_kernel<32, 3, __half, false, true, false, false>;
 }
 
 cudaError_t descent_config_tab(int, int, bool, const WalkArgs &wa, int sms, int *wpc, int *grid, size_t *smem)

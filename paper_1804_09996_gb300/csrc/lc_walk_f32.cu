@@ -9,8 +9,11 @@ cudaError_t walk_config_f32(int variant, int M1, bool fq, const WalkArgs &wa, si
 {
     return by_shape<float>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? launch_walk<T::M1, T::D1, float, T::FQ, false, true>(wa, per_warp, sms, want, wpc, grid, smem)
-                           : launch_walk<T::M1, T::D1, float, T::FQ, false, false>(wa, per_warp, sms, want, wpc, grid, smem);
+        const auto fn = wa.team > 1 ? (wa.beam > 1 ? launch_walk<T::M1, T::D1, float, T::FQ, false, true, true>
+                                                   : launch_walk<T::M1, T::D1, float, T::FQ, false, false, true>)
+                                    : (wa.beam > 1 ? launch_walk<T::M1, T::D1, float, T::FQ, false, true, false>
+                                                   : launch_walk<T::M1, T::D1, float, T::FQ, false, false, false>);
+        return fn(wa, per_warp, sms, want, wpc, grid, smem);
     });
 }
 
@@ -19,19 +22,24 @@ cudaError_t walk_run_f32(int variant, int M1, bool fq, const WalkArgs &wa, size_
 {
     return by_shape<float>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        return wa.beam > 1 ? run_walk<T::M1, T::D1, float, T::FQ, false, true>(wa, smem, wpc, grid, st, pdl)
-                           : run_walk<T::M1, T::D1, float, T::FQ, false, false>(wa, smem, wpc, grid, st, pdl);
+        const auto fn = wa.team > 1 ? (wa.beam > 1 ? run_walk<T::M1, T::D1, float, T::FQ, false, true, true>
+                                                   : run_walk<T::M1, T::D1, float, T::FQ, false, false, true>)
+                                    : (wa.beam > 1 ? run_walk<T::M1, T::D1, float, T::FQ, false, true, false>
+                                                   : run_walk<T::M1, T::D1, float, T::FQ, false, false, false>);
+        return fn(wa, smem, wpc, grid, st, pdl);
     });
 }
 
 // The walk instantiation a plan launches (for finding its node in a captured graph).
-const void *walk_fn_f32(int variant, int M1, bool fq, bool batch)
+const void *walk_fn_f32(int variant, int M1, bool fq, bool batch, bool team)
 {
     const void *fn = nullptr;
     by_shape<float>(variant, M1, fq, [&](auto t) {
         using T = decltype(t);
-        fn = batch ? (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, true>
-                   : (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, false>;
+        fn = team ? (batch ? (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, true, true>
+                           : (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, false, true>)
+                  : (batch ? (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, true, false>
+                           : (const void *)walk_kernel<T::M1, T::D1, float, T::FQ, false, false, false>);
         return cudaSuccess;
     });
     return fn;

@@ -58,18 +58,20 @@ def test_rows_with_repeated_ids(mix3k, beam):
 
 
 @pytest.mark.parametrize("name,u8", [("mix3k", False), ("opq3k", False), ("sift2k", True), ("odd2k", False)])
-@pytest.mark.parametrize("k,shortlist", [(10, 0), (40, 100)])
-def test_batch_size_does_not_matter(request, name, u8, k, shortlist):
-    # large batches (tiled rotation, one warp per re-ranked query) against small ones (direct
-    # rotation, teams of warps): the same bits for every query
+@pytest.mark.parametrize("k,shortlist,beam,prec,full", [(10, 0, 1, 0, 0), (40, 100, 4, 0, 0), (10, 0, 8, 1, 0), (10, 0, 1, 0, 1),
+                                                       (5, 0, 4, 0, 1)])
+def test_batch_size_does_not_matter(request, name, u8, k, shortlist, beam, prec, full):
+    # large batches (tiled rotation, one warp per query) against small ones (direct rotation,
+    # teams of warps in the walk and in the re-rank): the same bits for every query
     import torch
     ix, xb, xq = request.getfixturevalue(name)
     h = handle(name, ix)
     d = ix.d
     q = torch.from_numpy(np.ascontiguousarray(np.tile(xq, (4133 // len(xq) + 1, 1))[:4133], np.uint8 if u8 else np.float32)).cuda()
-    sp = lc.lc_default_search_params(k, 48, shortlist=shortlist)
+    sp = lc.lc_default_search_params(k, 48, shortlist=shortlist, lut_prec=prec, walk_full=full,
+                                     mode=lc.LC_MODE_BATCHED if beam > 1 else lc.LC_MODE_PLAIN, beam=beam)
     out = {}
-    for size in (4133, 601, 7):
+    for size in (4133, 701, 7):
         n = 4133 if size == 4133 else 3 * size
         ids = torch.empty((n, k), dtype=torch.int32, device="cuda")
         ds = torch.empty((n, k), dtype=torch.float32, device="cuda")
@@ -77,7 +79,7 @@ def test_batch_size_does_not_matter(request, name, u8, k, shortlist):
             lc.lc_search_ex(h, q[a:a + size], lc.LC_QUERY_U8 if u8 else lc.LC_QUERY_F32, size, sp, None, ids[a:a + size],
                             ds[a:a + size], None, torch.cuda.current_stream())
         out[size] = ids.cpu().numpy(), ds.cpu().numpy()
-    for size in (601, 7):
+    for size in (701, 7):
         n = 3 * size
         assert np.array_equal(out[size][0], out[4133][0][:n])
         assert np.array_equal(out[size][1].view(np.int32), out[4133][1][:n].view(np.int32))
