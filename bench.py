@@ -455,7 +455,6 @@ def measure_large(args, dev, flush, stream):
     ids = torch.empty((nq, k), dtype=torch.int32, device="cuda")
     dists = torch.empty((nq, k), dtype=torch.float32, device="cuda")
     stats = torch.empty((nq, 3), dtype=torch.int32, device="cuda")
-    lc.lc_profile(h, True)
     steps = max(5, args.steps // 2)
 
     def run(sp, n_steps):
@@ -463,15 +462,21 @@ def measure_large(args, dev, flush, stream):
             lc.lc_search(h, q, nq, sp, ids, dists, stats, stream)
         stream.synchronize()
         ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(n_steps)]
-        ph = []
         for e0, e1 in ev:
             with torch.cuda.stream(stream):
                 flush.sum(dtype=torch.int64)
                 e0.record(stream)
             lc.lc_search(h, q, nq, sp, ids, dists, stats, stream)
             e1.record(stream)
-            ph.append(lc.lc_profile_phases(h))
         torch.cuda.synchronize()
+        ph = []                                            # phases of serial, profiled steps
+        lc.lc_profile(h, True)
+        for _ in range(min(n_steps, 10)):
+            with torch.cuda.stream(stream):
+                flush.sum(dtype=torch.int64)
+            lc.lc_search(h, q, nq, sp, ids, dists, stats, stream)
+            ph.append(lc.lc_profile_phases(h))
+        lc.lc_profile(h, False)
         ms = float(np.mean([a.elapsed_time(b) for a, b in ev]))
         ph = np.mean(np.array(ph), axis=0)
         return dict(ms=ms, qps=nq / (ms / 1e3), walk_ms=float(ph[0] + ph[1] + ph[2]), refine_ms=float(ph[3]),
@@ -714,7 +719,6 @@ def main():
     stats = torch.empty((nq, 3), dtype=torch.int32, device="cuda")
     flush = torch.ones(256 << 20, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.Stream()
-    lc.lc_profile(h, True)
 
     def params(level, mode, prec=lc.LC_LUT_FP32, vlog=0, full=0):
         """Search parameters at one sweep level: efSearch, or (uneven workloads) the factor
@@ -733,7 +737,6 @@ def main():
         stream.synchronize()
         ev0 = [torch.cuda.Event(enable_timing=True) for _ in range(steps)]
         ev1 = [torch.cuda.Event(enable_timing=True) for _ in range(steps)]
-        ph = []
         barrier(ws)
         torch.cuda.synchronize()
         t0 = time.perf_counter()
@@ -743,10 +746,19 @@ def main():
                 ev0[s].record(stream)
             lc.lc_search_ex(h, q, qtype, nq, sp, de, ids, dists, stats, stream)
             ev1[s].record(stream)
-            ph.append(lc.lc_profile_phases(h))
         torch.cuda.synchronize()
         barrier(ws)
         wall = time.perf_counter() - t0
+        # the phases of a few more steps: a profiled search runs its kernels one after another
+        # (the timed ones overlap the re-rank with the end of the walk)
+        ph = []
+        lc.lc_profile(h, True)
+        for _ in range(min(steps, 10)):
+            with torch.cuda.stream(stream):
+                flush.sum(dtype=torch.int64)
+            lc.lc_search_ex(h, q, qtype, nq, sp, de, ids, dists, stats, stream)
+            ph.append(lc.lc_profile_phases(h))
+        lc.lc_profile(h, False)
         ms = max_over_ranks(float(np.mean([a.elapsed_time(b) for a, b in zip(ev0, ev1)])), ws)
         got = ids.cpu().numpy()
         ph = np.mean(np.array(ph), axis=0)
