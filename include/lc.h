@@ -115,7 +115,7 @@ typedef struct {
     int max_dist;    /* search-time cap T (Section 3.1): 0 = none; > 0: the level-0 search stops
                         before an expansion once T distances have been computed there */
     int warps;       /* walk queries in flight per thread block: 0 = as many as fit in shared
-                        memory (at most 24); 1..16 = at most that many.  Results do not depend
+                        memory (at most 20); 1..16 = at most that many.  Results do not depend
                         on it (a launch-shape knob for the autotuner) */
     int walk_full;   /* 0: the walk scores the level-1 code by ADC (the default reading of
                         Section 4.1); 1: it scores the full two-level decode q = c1 + c2 (each
@@ -124,8 +124,8 @@ typedef struct {
                         uniform level-1 split (M1 = 16 or 32 at d = 96, M1 = 64 at d = 128) */
     int order;       /* order in which the walk takes the queries (lc_search, lc_search_ex and the
                         server's launches; plans always use query order).  LC_ORDER_AUTO (0):
-                        ordered once the batch has at least twice as many queries as the GPU
-                        walks at once; LC_ORDER_NEVER: query order; LC_ORDER_ALWAYS: ordered.
+                        ordered once the batch has more queries than the GPU walks at once
+                        (twice as many where `warps` is set); LC_ORDER_NEVER: query order; LC_ORDER_ALWAYS: ordered.
                         Ordered: a first launch runs every query's upper-level descent, the
                         queries are sorted by decreasing distance to the node where it enters
                         level 0 (those tend to walk longest), and the level-0 searches run in

@@ -201,7 +201,6 @@ static void launch_rotate(const float *Q, const uint8_t *Q8, int64_t nq, int d, 
 // Within a bucket the order is whatever the atomics give; results do not depend on it.
 constexpr int ORDER_THREADS = 1024;
 constexpr int ORDER_BUCKETS = 2 * ORDER_THREADS;     // each thread sums two buckets
-constexpr int ORDER_MIN_ROUNDS = 2;                  // auto: queries >= 2 x warps in flight
 
 __device__ __forceinline__ int order_bucket(float x)
 {
@@ -779,10 +778,15 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     P.spill_tables = std::min<int64_t>(nq, (int64_t)P.grid * P.wpc);
     P.spill_elems = (size_t)P.spill_tables << P.spill_log;
     P.yq_elems = (size_t)nq * dv->d;
-    // ordered search: worth its two extra launches once every warp takes a few queries
+    // ordered search: worth its two extra launches once some walk takes a second query.  Query order
+    // against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500 queries, 550
+    // and 550 at 3,100, 643 and 561 at 3,600, 768 and 637 at 5,500; batched FP16 410 and 414, 464 and
+    // 419, 524 and 462 us at the last three.  With a set number of walks the line stays at two rounds
+    // (the scratch such a search was sized for)
+    const int64_t in_flight = (int64_t)P.grid * P.wpc;
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
                 (sp->order == LC_ORDER_ALWAYS ||
-                 (sp->order == LC_ORDER_AUTO && nq >= (int64_t)ORDER_MIN_ROUNDS * P.grid * P.wpc));
+                 (sp->order == LC_ORDER_AUTO && (sp->warps ? nq >= 2 * in_flight : nq > in_flight)));
     P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
     if (P.ordered) {
         // the descent launch: its own kernel, many more warps (no level-0 state)

@@ -21,9 +21,9 @@
 //     with a per-warp table in global memory behind it;
 //   - writes the shortlist (the R best of W, Section 4.1 two-stage search) or, without
 //     refinement, the top-k directly;
-//   - ordered search: a first launch (mode 1) runs only the upper-level descent of every query
-//     and records where it enters level 0; a second (mode 2) runs the level-0 searches from
-//     those entry nodes in the order the host sorted them (the queries whose entry node is
+//   - ordered search: descent_kernel runs only the upper-level descent of every query and
+//     records where it enters level 0; the walk (mode 2) runs the level-0 searches from those
+//     entry nodes in the order that order_kernel sorted them (the queries whose entry node is
 //     farthest from them first: they tend to walk longest, so the launch no longer ends with a
 //     few long walks on an otherwise idle GPU).  Each query's result is the same as in one
 //     launch (mode 0): the entry node and its distance are the ones the descent computes.
