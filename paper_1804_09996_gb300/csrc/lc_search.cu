@@ -778,28 +778,6 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     P.spill_tables = std::min<int64_t>(nq, (int64_t)P.grid * P.wpc);
     P.spill_elems = (size_t)P.spill_tables << P.spill_log;
     P.yq_elems = (size_t)nq * dv->d;
-    // ordered search: worth its two extra launches once some walk takes a second query.  Query order
-    // against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500 queries, 550
-    // and 550 at 3,100, 643 and 561 at 3,600, 768 and 637 at 5,500; batched FP16 410 and 414, 464 and
-    // 419, 524 and 462 us at the last three.  With a set number of walks the line stays at two rounds
-    // (the scratch such a search was sized for)
-    const int64_t in_flight = (int64_t)P.grid * P.wpc;
-    P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
-                (sp->order == LC_ORDER_ALWAYS ||
-                 (sp->order == LC_ORDER_AUTO && (sp->warps ? nq >= 2 * in_flight : nq > in_flight)));
-    P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
-    if (P.ordered) {
-        // the descent launch: its own kernel, many more warps (no level-0 state)
-        WalkArgs wd{};
-        wd.nq = nq;
-        wd.d = dv->d;
-        wd.M2P = dv->M2P;
-        ce = descent_config(P.form(), P.variant, dv->M1, P.full, wd, dv->num_sms, &P.dwpc, &P.dgrid, &P.dsmem);
-        if (ce != cudaSuccess) {
-            set_error("descent kernel configuration failed: %s", cudaGetErrorString(ce));
-            return LC_ERR_CUDA;
-        }
-    }
     if (rotate_tiled(nq, dv->d) &&
         cudaFuncSetAttribute(rotate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_PER_BLOCK) != cudaSuccess) {
         set_error("rotation kernel configuration failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -840,6 +818,32 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P.rw * 32, P.rsm);
         const int64_t teams = P.rw / P.rteam, need = (nq + teams - 1) / teams;
         P.rgrid = (int)std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * dv->num_sms);
+    }
+    // ordered search: worth its two extra launches once an eighth of the walks take a second query.
+    // Query order against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500
+    // queries, 550 and 550 at 3,100, 643 and 561 at 3,600, 768 and 637 at 5,500; batched FP16 410 and
+    // 414, 464 and 419, 524 and 462 us at the last three; without re-rank 297 and 316 at 3,100, 380
+    // and 340 at 3,600.  From two rounds on where the number of walks is set (the scratch such a
+    // search was sized for), and where the re-rank, by teams and with C2 through L1, is the longer
+    // part: it would take its queries one warp each (d = 128, R = 100, 3,600 queries: 702 and 738 us;
+    // 878 and 839 at 4,500)
+    const int64_t in_flight = (int64_t)P.grid * P.wpc;
+    const bool late = sp->warps || (P.refine && P.rteam > 1 && !P.rboth);
+    P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
+                (sp->order == LC_ORDER_ALWAYS ||
+                 (sp->order == LC_ORDER_AUTO && (late ? nq >= 2 * in_flight : nq >= in_flight + in_flight / 8)));
+    P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
+    if (P.ordered) {
+        // the descent launch: its own kernel, many more warps (no level-0 state)
+        WalkArgs wd{};
+        wd.nq = nq;
+        wd.d = dv->d;
+        wd.M2P = dv->M2P;
+        ce = descent_config(P.form(), P.variant, dv->M1, P.full, wd, dv->num_sms, &P.dwpc, &P.dgrid, &P.dsmem);
+        if (ce != cudaSuccess) {
+            set_error("descent kernel configuration failed: %s", cudaGetErrorString(ce));
+            return LC_ERR_CUDA;
+        }
     }
     *pl = P;
     return LC_OK;
