@@ -459,6 +459,7 @@ __global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(a.list + i) : "memory");
                 if (e < 0) continue;                 // (never: every walk leaves its entry)
             }
+            __syncwarp();                            // lane 0's acquire before every lane's reads of the shortlist
             q = e;
         } else if (it >= a.nq) {
             break;

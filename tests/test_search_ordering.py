@@ -1,0 +1,22 @@
+"""Memory ordering between the kernels of one search, read from the sources (a missing ordering
+does not show in results, so no run can test for it)."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1804_09996_gb300", "csrc")
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_rerank_orders_the_shortlist_after_the_walk_that_wrote_it():
+    # The re-rank of an ordered search runs while walks still write.  One lane acquires the entry
+    # of an ended walk; a shuffle hands the query to the others but orders no memory, so a warp
+    # barrier has to stand between the acquire and the reads of the shortlist.
+    body = source("lc_search.cu").split("refine_kernel(const RefineArgs a)")[1]
+    acquire, read = body.index("ld.acquire.gpu"), body.index("a.shortlist")
+    assert acquire < read
+    last_shuffle = body.rindex("__shfl_sync(FULL, e, 0)", acquire, read)
+    assert "__syncwarp()" in body[last_shuffle:read]
