@@ -222,8 +222,19 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_kernel(const float *key, 
     }
     for (int i = t; i < ORDER_BUCKETS; i += ORDER_THREADS) pos[i] = 0;
     __syncthreads();
-#pragma unroll 8
-    for (int64_t i = t; i < n; i += ORDER_THREADS) atomicAdd(&pos[order_bucket(__ldg(key + i))], 1u);
+    // plain loads (the descent that wrote the keys may have run when this kernel started), eight of
+    // a thread in flight at once
+    auto each_key = [&](auto f) {
+        for (int64_t i0 = t; i0 < n; i0 += 8 * ORDER_THREADS) {
+            float k[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) k[u] = i0 + u * ORDER_THREADS < n ? key[i0 + u * ORDER_THREADS] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (i0 + u * ORDER_THREADS < n) f(i0 + u * ORDER_THREADS, order_bucket(k[u]));
+        }
+    };
+    each_key([&](int64_t, int b) { atomicAdd(&pos[b], 1u); });
     __syncthreads();
     // thread t owns buckets b0 = 2047 - 2t and b0 - 1 (ranks 2t and 2t + 1 in decreasing order)
     const int b0 = ORDER_BUCKETS - 1 - 2 * t, b1 = b0 - 1;
@@ -252,11 +263,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) order_kernel(const float *key, 
     pos[b0] = ex;                                     // only this thread reads or writes b0, b1
     pos[b1] = ex + c0;
     __syncthreads();
-#pragma unroll 8
-    for (int64_t i = t; i < n; i += ORDER_THREADS) {
-        const uint32_t p = atomicAdd(&pos[order_bucket(__ldg(key + i))], 1u);
-        order[p] = (int32_t)i;
-    }
+    each_key([&](int64_t i, int b) { order[atomicAdd(&pos[b], 1u)] = (int32_t)i; });
 }
 
 // Per-query ADC tables on the tensor cores (table_kernel, search form LC_LUT_TABLE), for the

@@ -145,6 +145,9 @@ struct WalkArgs {
 // free (pdl_launch), and wait for the previous one to have ended (pdl_wait) once their codebooks
 // are in shared memory, before they touch anything it writes.  Each lets the next one start only
 // after its own wait, so a kernel that runs has everything of the kernels before the one ahead of it.
+// What the kernel ahead writes (entry nodes, distances and order of an ordered search) is read by
+// plain loads: the read-only path (__ldg) is for data that no one writes while the reader's grid
+// lives, and its loads may be moved ahead of the wait.
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -1148,7 +1151,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             qi = ctl[0];
         }
         if (qi >= a.nq) break;
-        const int64_t q = a.order ? (int64_t)__ldg(a.order + qi) : qi;
+        const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
         V.spill = a.spill + ((a.spill_tables >= a.nq ? qi : gwarp) << a.spill_log);
         // this query's ef' = max(ef, k)
         const int efp = a.efq ? max(min(max(__ldg(a.efq + q), 1), a.efp), a.k) : a.efp;
@@ -1212,9 +1215,9 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
         const int B = BATCH ? a.beam : 1;  // level-0 expansions per step
         if (a.mode == 2) {
             // level 0 from the entry node the descent launch recorded (as at its end below)
-            cur = __ldg(a.seed + q);
-            dcur = __ldg(a.seed_d + q);
-            n_up = __ldg(a.seed_up + q);
+            cur = a.seed[q];
+            dcur = a.seed_d[q];
+            n_up = a.seed_up[q];
             phase = 2;
             if (lane == 0) W[0] = walk_key(dcur, cur);
             V.first(a.vt, cur, lane);

@@ -20,3 +20,13 @@ def test_rerank_orders_the_shortlist_after_the_walk_that_wrote_it():
     assert acquire < read
     last_shuffle = body.rindex("__shfl_sync(FULL, e, 0)", acquire, read)
     assert "__syncwarp()" in body[last_shuffle:read]
+
+
+def test_read_only_loads_take_nothing_that_an_earlier_kernel_of_the_search_writes():
+    # A kernel of a search may start while the one ahead still writes, and the read-only load path
+    # is only for data that stays unwritten while the reading grid lives.
+    written = r"\b(a\.(seed|seed_d|seed_up|order|yq|yq_in|shortlist|list|done_list)|key|yrot|sl)\b"
+    for name in ("lc_walk.cuh", "lc_search.cu"):
+        loads = re.findall(r"__ldg\(([^;]*)", source(name))
+        assert loads
+        assert not [x for x in loads if re.match(written, x.strip())], name
