@@ -469,20 +469,33 @@ __device__ __forceinline__ void pair_full(const CT *C1s, const CT *C2, int d, in
                                           const uint8_t *rb, const LaneGeo<M1, D1> &g, int k, float &s0, float &s1)
 {
     constexpr int DMAX = LaneGeo<M1, D1>::DMAX;
-    float x0[DMAX], x1[DMAX], z0[DMAX], z1[DMAX];
-    load_row<M1, D1, CT>(C1s, d, c0, g, k, x0);
-    load_row<M1, D1, CT>(C1s, d, c1, g, k, x1);
-    load_row2<M1, D1, CT, TWO>(C2, d, ra, g, k, z0);
-    load_row2<M1, D1, CT, TWO>(C2, d, rb, g, k, z1);
     unsigned long long acc = 0ull;
-#pragma unroll
-    for (int u = 0; u < DMAX; u++) {
-        if (D1 == 0 && u >= g.maxlen) continue;
+    auto add = [&](int u, float x0, float x1, float z0, float z1) {
         const unsigned long long yy = pack2(g.y[k][u], g.y[k][u]);
         unsigned long long v, df;
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pack2(x0[u], x1[u])), "l"(pack2(z0[u], z1[u])));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(pack2(x0, x1)), "l"(pack2(z0, z1)));
         asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(df) : "l"(yy), "l"(v));
         asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(acc) : "l"(df), "l"(acc));
+    };
+    if constexpr (DMAX <= 6) {
+        float x0[DMAX], x1[DMAX], z0[DMAX], z1[DMAX];
+        load_row<M1, D1, CT>(C1s, d, c0, g, k, x0);
+        load_row<M1, D1, CT>(C1s, d, c1, g, k, x1);
+        load_row2<M1, D1, CT, TWO>(C2, d, ra, g, k, z0);
+        load_row2<M1, D1, CT, TWO>(C2, d, rb, g, k, z1);
+#pragma unroll
+        for (int u = 0; u < DMAX; u++)
+            if (D1 > 0 || u < g.maxlen) add(u, x0[u], x1[u], z0[u], z1[u]);
+    } else {
+        // (uneven splits) coordinate by coordinate: rows of up to 16 coordinates would not fit the
+        // registers; those past the lane's own length count 0
+        const CT *p0 = C1s + c0 * d + g.off[k], *p1 = C1s + c1 * d + g.off[k], *q = C2 + g.off[k];
+#pragma unroll
+        for (int u = 0; u < DMAX; u++) {
+            if (u >= g.maxlen) break;
+            if (u < g.len[k])
+                add(u, to_f(p0[u]), to_f(p1[u]), c2_at(q + (int)ra[g.sub2(k, u)] * d + u), c2_at(q + (int)rb[g.sub2(k, u)] * d + u));
+        }
     }
     unpack2(acc, s0, s1);
 }
@@ -500,6 +513,12 @@ __device__ __forceinline__ void pair_full(const CT *C1s, const CT *C2, int d, in
 // waiting for instructions).
 __host__ __device__ constexpr int slot_block(int M1) { return M1 == 16 ? 16 : 8; }
 
+// Full walk: whether C2 is read only for nodes that are there (see block_terms): in FP32, but for
+// 96/32, whose whole blocks of eight keep more reads in flight: 338 against 391 us at 1,000 queries
+// and 70.4 against 71.8 ms for a GPU-assisted add of 40,000 vectors (from some 1,500 queries on node
+// by node is faster: 588 and 483 us at 2,000, 3,816 and 2,320 at 20,000).
+__host__ __device__ constexpr bool node_by_node(int M1, int D1, int es) { return es == 4 && !(M1 == 32 && D1 == 3); }
+
 template <int M1>
 __device__ __forceinline__ int lane_block(int lane)
 {
@@ -513,12 +532,12 @@ __device__ __forceinline__ int chunk_slot(int lane)
     return lane_block<M1>(lane) * slot_block(M1) + (M1 == 16 ? 2 * s3 + (lane >> 4) : s3);
 }
 
-// The eight values of this lane for the block staged at `stage` (residual rows at `stage2`).
-// Slots past the nodes staged hold stale bytes, which are codes all the same; their totals are
-// not used.  TAB: C1s is the query's ADC table [256][M1] (FP16): the term of code c is its entry
+// The eight values of this lane for the block staged at `stage` (residual rows at `stage2`), whose
+// first n >= 1 slots hold nodes (n may be more than a block).  The slots behind them hold stale
+// bytes, which are codes all the same; their totals are not used.  TAB: C1s is the query's ADC table [256][M1] (FP16): the term of code c is its entry
 // [c][lane].
 template <int M1, int D1, typename CT, bool FQ, bool TAB, bool TWO>
-__device__ __forceinline__ void block_terms(const CT *C1s, const uint8_t *stage, const uint8_t *stage2, int d,
+__device__ __forceinline__ void block_terms(const CT *C1s, const uint8_t *stage, const uint8_t *stage2, int n, int d,
                                             const LaneGeo<M1, D1> &g, int lane, const CT *C2, int M2P, float (&v)[8])
 {
     // node of value i for this lane, and its code in sub-space j
@@ -528,6 +547,37 @@ __device__ __forceinline__ void block_terms(const CT *C1s, const uint8_t *stage,
         static_assert(M1 == 32 && !FQ, "the table form is built for 32 sub-spaces");
 #pragma unroll
         for (int i = 0; i < 8; i++) v[i] = to_f(C1s[(int)stage[slot(i) * M1 + lane] * M1 + lane]);
+    } else if constexpr (FQ && node_by_node(M1, D1, (int)sizeof(CT))) {
+        // C2 comes through the cache, which bounds this form, so only nodes that are there read it: the
+        // lanes take the same two nodes at a time (with M1 = 16 two per half-warp), up to the last, and
+        // the values change places afterwards.  A step has about six new nodes, and a block's other
+        // slots would read C2 for nothing, each lane for another node (20,000 queries, ef 64, on 20,000
+        // x 96 with M1 = 16: 6,894 us with whole blocks, 2,136 now; x 128 with M1 = 64: 6,532 and 3,902;
+        // x 100 with M1 = 16, where whole blocks also spill: 11,671 and 3,791).
+        auto node = [&](int i) { return min(M1 == 16 ? 2 * i + h : i, n - 1); };
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            v[i] = v[i + 1] = 0.f;
+            if ((M1 == 16 ? 2 * i : i) >= n) continue;
+            const uint8_t *ca = stage + node(i) * M1, *cb = stage + node(i + 1) * M1;
+            const uint8_t *ra = stage2 + node(i) * M2P, *rb = stage2 + node(i + 1) * M2P;
+            pair_full<M1, D1, CT, TWO>(C1s, C2, d, ca[j], cb[j], ra, rb, g, 0, v[i], v[i + 1]);
+            if (M1 == 64) {
+                float u0, u1;
+                pair_full<M1, D1, CT, TWO>(C1s, C2, d, ca[32 + j], cb[32 + j], ra, rb, g, LaneGeo<M1, D1>::NSUB - 1, u0, u1);
+                v[i] += u0;
+                v[i + 1] += u1;
+            }
+        }
+#pragma unroll
+        for (int b = 1; b < 8; b *= 2)
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                if (!(i & b)) {
+                    const float lo = v[i], hi = v[i | b];
+                    v[i] = s3 & b ? hi : lo;
+                    v[i | b] = s3 & b ? lo : hi;
+                }
     } else if constexpr (FQ) {
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
@@ -649,8 +699,9 @@ __device__ __forceinline__ float score_staged(const CT *C1s, const uint8_t *stag
     float r = 0.f;
     auto terms = [&](int b, float (&v)[8]) {
         const uint8_t *st = stage + b * SB * M1, *st2 = stage2 + b * SB * M2P;
-        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, TAB, false>(C1s, st, st2, d, g, lane, C2, M2P, v);
-        else block_terms<M1, D1, CT, FQ, TAB, true>(C1s, st, st2, d, g, lane, C2, M2P, v);
+        const int n = nf - b * SB;
+        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, TAB, false>(C1s, st, st2, n, d, g, lane, C2, M2P, v);
+        else block_terms<M1, D1, CT, FQ, TAB, true>(C1s, st, st2, n, d, g, lane, C2, M2P, v);
     };
 #pragma unroll 1
     for (int b = 0; b * SB < nf; b += PAIR ? 2 : 1) {
@@ -1091,8 +1142,8 @@ __device__ __forceinline__ void score_team(const CT *C1s, uint8_t *stage, const 
         copy_wait();
         __syncwarp();
         float v[8];
-        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, false, false>(C1s, st, st2, d, g, lane, C2, M2P, v);
-        else block_terms<M1, D1, CT, FQ, false, true>(C1s, st, st2, d, g, lane, C2, M2P, v);
+        if (FQ && D1 > 2 && !g.two) block_terms<M1, D1, CT, FQ, false, false>(C1s, st, st2, n - b * SB, d, g, lane, C2, M2P, v);
+        else block_terms<M1, D1, CT, FQ, false, true>(C1s, st, st2, n - b * SB, d, g, lane, C2, M2P, v);
         const float t = reduce_block<M1>(v);
         if (lane_block<M1>(lane) == 0 && b * SB + node < n) dist[b * SB + node] = t;
         __syncwarp();
