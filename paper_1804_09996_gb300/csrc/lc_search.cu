@@ -404,8 +404,11 @@ __host__ __device__ inline size_t refine_keys(int R) { return (size_t)((R + 1) &
 // shared memory (copied with all loads in flight; d*4 bytes is a multiple of 128 at d = 96 and
 // 128, so lane t reading coordinate t of any centroid hits bank t mod 32); otherwise only C1 does
 // and C2 is read through the cache.  DU: coordinates per lane, d <= 32 DU (CHECK: d < 32 DU).
+// One block per SM is said to the compiler: without it, it keeps the forms with C2 through the cache
+// to 64 registers, which do not hold a candidate's reads of C2 in flight (20,000 queries, d = 128,
+// R = 10: 520 us, 408 with it; with a product codebook of 8 blocks 626 and 337).
 template <bool C2_SHARED, int DU, bool PROD, bool CHECK>
-__global__ void __launch_bounds__(16 * 32) refine_kernel(const RefineArgs a)
+__global__ void __launch_bounds__(16 * 32, 1) refine_kernel(const RefineArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
