@@ -834,12 +834,11 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     // Query order against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500
     // queries, 550 and 550 at 3,100, 643 and 561 at 3,600, 768 and 637 at 5,500; batched FP16 410 and
     // 414, 464 and 419, 524 and 462 us at the last three; without re-rank 297 and 316 at 3,100, 380
-    // and 340 at 3,600.  From two rounds on where the number of walks is set (the scratch such a
-    // search was sized for), and where the re-rank, by teams and with C2 through L1, is the longer
-    // part: it would take its queries one warp each (d = 128, R = 100, 3,600 queries: 702 and 738 us;
-    // 878 and 839 at 4,500)
+    // and 340 at 3,600.  On 12,000 x 128 (M1 = 64, C2 through the cache): 396 and 358 us at 2,700, 442 and
+    // 366 at 3,600; with R = 100 884 and 836, 1,104 and 1,024.  From two rounds on where the number of
+    // walks is set (the scratch such a search was sized for)
     const int64_t in_flight = (int64_t)P.grid * P.wpc;
-    const bool late = sp->warps || (P.refine && P.rteam > 1 && !P.rboth);
+    const bool late = sp->warps;
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
                 (sp->order == LC_ORDER_ALWAYS ||
                  (sp->order == LC_ORDER_AUTO && (late ? nq >= 2 * in_flight : nq >= in_flight + in_flight / 8)));
@@ -921,8 +920,12 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     // large batches: the re-rank takes the queries as their walks end, on the SMs that have no more
     // (at 10k queries an SM is idle for a tenth of the walk launch while the longest walks end, and
     // the re-rank mostly fits into that: 721 -> 654 us for the batched FP16 search, 857 -> 781 us for
-    // the plain one, launch latencies included)
-    const bool overlap = P.ordered && P.refine && !profile;
+    // the plain one, launch latencies included).  Not a re-rank that reads C2 through L1: started while
+    // the walk is there, an SM keeps the walk's split of its memory (228 KB shared, 28 KB of L1) where the
+    // re-rank alone gets 60 KB of L1, and takes 702 us in place of 395 (20,000 queries, d = 128, R = 10).
+    // It is launched when the walk has ended, by teams where those are faster (whole searches of 20,000
+    // queries at d = 128: 1,848 -> 1,592 us, with beam 2 and R = 30 3,051 -> 2,254)
+    const bool overlap = P.ordered && P.refine && P.rboth && !profile;
     if (ce == cudaSuccess && P.tab) {
         // the batch's ADC tables on the tensor cores, from y'
         table_kernel<<<(unsigned)((nq + TAB_WARPS * 8 - 1) / (TAB_WARPS * 8)), TAB_WARPS * 32, 0, st>>>(
@@ -989,7 +992,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
             ra.head = wa.done_tail + 1;
         }
         auto kern = refine_kernel_for(P.rboth, dv->d, dv->bM > 1);
-        ce = launch(kern, P.rgrid, P.rw * 32, P.rsm, st, !profile, ra);
+        ce = launch(kern, P.rgrid, P.rw * 32, P.rsm, st, P.rboth && !profile, ra);
         if (ce != cudaSuccess) {
             set_error("refine kernel launch failed: %s", cudaGetErrorString(ce));
             return LC_ERR_CUDA;
