@@ -125,8 +125,7 @@ typedef struct {
     int order;       /* order in which the walk takes the queries (lc_search, lc_search_ex and the
                         server's launches; plans always use query order).  LC_ORDER_AUTO (0):
                         ordered once the batch has an eighth more queries than the GPU walks
-                        at once (twice as many where `warps` is set); LC_ORDER_NEVER: query
-                        order; LC_ORDER_ALWAYS: ordered.
+                        at once; LC_ORDER_NEVER: query order; LC_ORDER_ALWAYS: ordered.
                         Ordered: a first launch runs every query's upper-level descent, the
                         queries are sorted by decreasing distance to the node where it enters
                         level 0 (those tend to walk longest), and the level-0 searches run in

@@ -835,13 +835,11 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     // queries, 550 and 550 at 3,100, 643 and 561 at 3,600, 768 and 637 at 5,500; batched FP16 410 and
     // 414, 464 and 419, 524 and 462 us at the last three; without re-rank 297 and 316 at 3,100, 380
     // and 340 at 3,600.  On 12,000 x 128 (M1 = 64, C2 through the cache): 396 and 358 us at 2,700, 442 and
-    // 366 at 3,600; with R = 100 884 and 836, 1,104 and 1,024.  From two rounds on where the number of
-    // walks is set (the scratch such a search was sized for)
+    // 366 at 3,600; with R = 100 884 and 836, 1,104 and 1,024.  Where the number of walks is set, 8 per
+    // block: 329 and 303 us at 1,459, 382 and 297 at 1,824 (20,000 x 96)
     const int64_t in_flight = (int64_t)P.grid * P.wpc;
-    const bool late = sp->warps;
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
-                (sp->order == LC_ORDER_ALWAYS ||
-                 (sp->order == LC_ORDER_AUTO && (late ? nq >= 2 * in_flight : nq >= in_flight + in_flight / 8)));
+                (sp->order == LC_ORDER_ALWAYS || (sp->order == LC_ORDER_AUTO && nq >= in_flight + in_flight / 8));
     P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
     if (P.ordered) {
         // the descent launch: its own kernel, many more warps (no level-0 state)

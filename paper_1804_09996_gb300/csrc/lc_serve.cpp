@@ -171,14 +171,16 @@ lc_status plan_batch(lc_server *s, Batch &b)
     }
     b.sp.ef = efb;                              // the bound of the per-query efSearch
     // a lone request whose walks in flight would need more visited tables than the budget holds
-    // runs with fewer walks at a time (results do not depend on it)
-    for (int warps = b.reqs[0]->sp.warps;;) {
-        b.sp.warps = warps;
+    // runs with fewer walks at a time, and without the ordered search's scratch if that is still
+    // too much (results do not depend on either)
+    for (;;) {
         lc_status rs = lc::plan_search(s->dv, b.nq, &b.sp, &b.plan, true);
         if (rs != LC_OK) return rs;
         layout(b, s->dv->d);
-        if (b.need <= s->budget || b.reqs.size() > 1 || b.plan.wpc == 1) return LC_OK;
-        warps = b.plan.wpc > 16 ? 16 : b.plan.wpc / 2;
+        if (b.need <= s->budget || b.reqs.size() > 1) return LC_OK;
+        if (b.plan.wpc > 1) b.sp.warps = b.plan.wpc > 16 ? 16 : b.plan.wpc / 2;
+        else if (b.plan.ordered) b.sp.order = LC_ORDER_NEVER;
+        else return LC_OK;
     }
 }
 
