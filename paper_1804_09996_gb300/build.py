@@ -53,7 +53,8 @@ def build(verbose: bool = False, force: bool = False) -> str:
         else:
             cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
             # no multiply-add contraction: the host build gives the same bits on x86 and Arm, and
-            # the device codeword assignment reproduces it exactly
+            # the device codeword assignment reproduces it exactly (the .cu files' host code is compiled
+            # without this: the device encoder's centroid norms may be contracted on Arm)
             cmd = ["g++", "-std=c++17", "-O3", "-ffp-contract=off", "-fPIC", "-pthread", "-Wall", "-I", cuda_inc,
                    "-c", src, "-o", obj]
         jobs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))

@@ -1148,7 +1148,7 @@ lc_status build_add(lc_index *ix, const float *x, int64_t n)
     std::vector<float> xr((size_t)n * d);
     std::vector<uint8_t> nc1((size_t)n * p.M1), nc2((size_t)n * p.M2);
     if (p.build_gpu) {
-        // rotation and both code levels on the device (the host's arithmetic, the host's codes)
+        // rotation and both code levels on the device (the host's arithmetic but for the centroids' norms)
         lc_status rs = build_gpu_encode(ix, x, n, xr.data(), nc1.data(), nc2.data());
         if (rs != LC_OK) return rs;
     } else {

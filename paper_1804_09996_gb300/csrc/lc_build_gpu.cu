@@ -484,7 +484,9 @@ lc_status build_gpu_assign(lc_index *ix, const float *xr, int64_t first, int64_t
 // Encoding of the vectors being added (rotation, level-1 PQ, residual, level-2 PQ), in the host
 // build's float arithmetic (the rotation sums R[t][u] x_u over u in order; each centroid's
 // score is ||c||^2 plus (-2 x_t) c_t over t in order; the first minimum wins; no multiply-add
-// contraction), so the codes are the host's.
+// contraction).  The codes are the host's up to near-ties: the norms are summed by this file's host
+// code, whose compiler may contract them on machines with a fused multiply-add (on aarch64 it does:
+// one of the 120,000 level-2 codes of tests/test_gpu_build_codes.py).
 __global__ void rotate_exact_kernel(const float *X, int64_t n, int d, const float *RT, float *Y)
 {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * d; e += (int64_t)gridDim.x * blockDim.x) {
@@ -545,7 +547,8 @@ lc_status build_gpu_encode(lc_index *ix, const float *x, int64_t n, float *xr, u
             set_error("device encoding needs sub-spaces of at most 16 dimensions");
             return LC_ERR_ARG;
         }
-    // transposed rotation and squared centroid norms exactly as the host computes them
+    // transposed rotation, and squared centroid norms summed in the host build's order (maybe contracted,
+    // see above)
     std::vector<float> RT((size_t)d * d), cn1((size_t)M1 * 256, 0.f), cn2((size_t)M2 * 256, 0.f);
     for (int t = 0; t < d; t++)
         for (int u = 0; u < d; u++) RT[(size_t)u * d + t] = ix->R[(size_t)t * d + u];
