@@ -1356,7 +1356,7 @@ __global__ void __launch_bounds__(walk_threads(D1, FQ)) walk_kernel(const WalkAr
             uint32_t bd = ~0u, bi = ~0u;
             const uint64_t wmax = phase == 2 && wn == efp ? W[wn - 1] : ~0ull;
             int nc = 0;
-            if constexpr (TEAM) {
+            if (TEAM && ns > 0) {                          // (0 would tell the team that the walk has ended)
                 if (lane == 0) ctl[1] = ns;
                 team_bar();
                 score_team<M1, D1, CT, FQ>(C1s, stage, a.codes1, a.codes2b, a.M2P, slot, ns, d, g, lane, 0, team, C2, dist);

@@ -30,3 +30,11 @@ def test_read_only_loads_take_nothing_that_an_earlier_kernel_of_the_search_write
         loads = re.findall(r"__ldg\(([^;]*)", source(name))
         assert loads
         assert not [x for x in loads if re.match(written, x.strip())], name
+
+
+def test_a_team_is_told_of_no_empty_step():
+    # The walk hands its helpers the number of nodes to score, and 0 says that the walk has ended: a
+    # row without neighbours (the top level, mostly) must not be announced.
+    body = source("lc_walk.cuh").split("walk_kernel(const WalkArgs a)")[1]
+    announce = body.index("ctl[1] = ns")
+    assert "ns > 0" in body[body.rindex("if", 0, body.rindex("{", 0, announce)):announce]
