@@ -432,7 +432,7 @@ lc_status build_gpu_assign(lc_index *ix, const float *xr, int64_t first, int64_t
         }
     }
     double *dW = nullptr;
-    if (!dupload(dv->B, ix->B) || !dupload(dW, W)) {   // trained after the graph
+    if (!dupload(dW, W)) {
         cfree(dW);
         set_error("upload of the regression codebook failed");
         return LC_ERR_OOM;
