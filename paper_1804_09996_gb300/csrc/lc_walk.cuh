@@ -151,7 +151,8 @@ struct WalkArgs {
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launches kern on st; pdl: it may start before the kernel queued ahead of it has ended.
+// Launches kern on st; pdl: it may start before the kernel queued ahead of it has ended.  A launch
+// that fails leaves no error behind for the next call to find.
 template <typename... P, typename... A>
 static cudaError_t launch(void (*kern)(P...), int64_t grid, int block, size_t smem, cudaStream_t st, bool pdl, A... args)
 {
@@ -165,7 +166,9 @@ static cudaError_t launch(void (*kern)(P...), int64_t grid, int block, size_t sm
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 constexpr int MAX_WALK_WARPS = 20;       // warps (queries in flight) per CTA
