@@ -33,7 +33,9 @@ struct LinkDev {
 // grow() for the buffers of the batches, which get larger one by one until batch_max: half as
 // much again as needed, so a build reallocates a few times and not once per batch (cudaMalloc
 // and cudaFree wait for the device: the searches' start took 57 ms of a 60,000-vector add's
-// 240 ms, and the whole add takes 213 ms with it).
+// 240 ms, and the whole add takes 213 ms with it).  The buffers go at the end of the add, but for the
+// searches' visited tables and order scratch, which are lc_search's own and stay with the index: up to
+// half as much again as the largest batch needed (tens of MB).
 template <class T>
 static bool grow_batch(T *&p, size_t &cap, size_t need)
 {

@@ -30,7 +30,7 @@ struct DeviceIndex {
     float *yq = nullptr; size_t yq_cap = 0;
     int32_t *shortlist = nullptr; size_t sl_cap = 0;
     int32_t *spill = nullptr; size_t spill_cap = 0;
-    int32_t *ord = nullptr; size_t ord_cap = 0;       // ordered search: 4 words per query
+    int32_t *ord = nullptr; size_t ord_cap = 0;       // ordered search: 5 words per query, 2 more
     uint16_t *tab = nullptr; size_t tab_cap = 0;      // table form: FP16 ADC tables [nq][256][32]
     int32_t *status = nullptr;
     unsigned long long *counter = nullptr;
@@ -97,10 +97,10 @@ inline bool grow(T *&p, size_t &cap, size_t need)
 //     identifies the id exactly.  An id whose bucket is full (or whose tag is 0) goes to a small table
 //     of ids in shared memory (2^stash_log entries) and, once that is three quarters full, to the
 //     global table.  Half the bytes of the ids per entry: a walk's table takes 4.5 KB and not 8,
-//     so that up to 24 walks fit on an SM and not 16.
+//     so that 20 walks fit on an SM and not 16.
 //   tag = 0: four 32-bit ids (plus one) per bucket, a full bucket continuing in the next, the
-//     global table behind; for indexes too large for the tags and for the table sizes that a
-//     caller asks for.
+//     global table behind; for indexes too large for the tags (more than 2^25 ids, 2^24 at the smaller
+//     limits) and for the table sizes that a caller asks for, also where they are the automatic ones.
 struct VisitTab {
     int tag, bb, tb, stash_log;
     uint32_t mul, bytes;           // multiplier, bytes of the buckets
@@ -138,15 +138,16 @@ struct SearchScratch {
     int32_t *spill = nullptr;            // [spill_tables][2^spill_log]
     uint16_t *tab = nullptr;             // table form: [nq][256][32] FP16
     int32_t *ord = nullptr;              // ordered search: entry node, upper evaluations, queue
-                                         // order (int32) and entry distance (float), [nq] each
+                                         // order (int32), entry distance (float) and the list of
+                                         // ended walks (int32), [nq] each, then its two heads
     int32_t *status = nullptr;           // 1 word
     unsigned long long *counter = nullptr;
 };
 
 lc_status upload(lc_index *ix);
 
-// allow_order: the caller provides the ordered search's scratch (lc_search / lc_search_ex do;
-// plans, served requests and the build's searches walk in query order).
+// allow_order: the caller provides the ordered search's scratch (lc_search / lc_search_ex, the server
+// and the build's searches do; plans walk in query order).
 lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params *sp, SearchPlan *pl,
                       bool allow_order = false);
 // Queues the walk (and refinement) on `st`; q, ids, dists, stats are device pointers.

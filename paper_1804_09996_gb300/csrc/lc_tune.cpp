@@ -154,7 +154,8 @@ lc_status autotune(lc_index *ix, const float *q, int64_t n, const int32_t *gt, c
             }
         }
     }
-    // stage 2: launch shape for the chosen parameters (results unchanged)
+    // stage 2: launch shape for the chosen parameters (results unchanged).  A table size that is asked
+    // for is held as ids (lc.h), so it wins only where the automatic tags are too wide or too small
     const lc_search_params chosen = out->sp;
     for (int vlog : {0, 10, 11, 12}) {
         for (int warps : {0, 4, 8, 12}) {

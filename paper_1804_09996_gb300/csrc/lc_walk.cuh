@@ -60,7 +60,10 @@ inline VisitTab visit_tab(int64_t n, int hash_log, bool want_tag)
     for (int h = hash_log; want_tag && h <= hash_log + 1; h++) {
         const int bb = h - 3;                             // 8 tags per bucket
         nb = nb <= bb ? bb + 1 : nb;
-        if (nb - bb > 16) continue;                       // one more bit of buckets: as large as with ids
+        // Tags of more than 16 bits: one more bit of buckets, which with the stash takes an eighth more
+        // than ids (2^11 limits: 9 KB and 8) but is probed once and without branches (8.4M ids, limits
+        // of 2^10, 10,000 queries: 553 us against 670 with ids, batched FP16 472 and 533).
+        if (nb - bb > 16) continue;
         v.tag = 1;
         v.bb = bb;
         v.tb = nb - bb;
@@ -293,7 +296,6 @@ __device__ __forceinline__ void warp_best(uint32_t dist, uint32_t id, uint32_t *
 
 // Lane bits in the order partial distances are combined: 3, 2, 1, 0, then 4.
 __host__ __device__ constexpr int comb_bit(int k) { return k < 4 ? 3 - k : 4; }
-__host__ __device__ constexpr int ilog2c(int s) { return s <= 1 ? 0 : 1 + ilog2c(s >> 1); }
 
 // The lane bits of the first LS combinations, the first one most significant.
 __device__ __forceinline__ int slot_of_lane(int lane, int LS)
@@ -511,7 +513,7 @@ __device__ __forceinline__ void pair_full(const CT *C1s, const CT *C2, int d, in
 // lower half and sends its upper one, without selects, and ends with node s3.  A lane keeps
 // the total of one node per chunk of 32: node chunk_slot(lane).
 // Blocks of eight in a rolled loop, and not one unrolled pass over 16 or 32 nodes: fewer
-// registers (24 warps per SM leave 80 each), no work past the last block, and code that stays in
+// registers (20 warps per SM leave 102 each), no work past the last block, and code that stays in
 // the instruction cache (the unrolled full-decode scoring lost two thirds of its stall cycles
 // waiting for instructions).
 __host__ __device__ constexpr int slot_block(int M1) { return M1 == 16 ? 16 : 8; }
@@ -1121,8 +1123,6 @@ __device__ __forceinline__ void load_codebooks(const WalkArgs &a, unsigned char 
     pdl_launch();
 }
 
-// TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
-// [256][M1] (FP16, built by table_kernel) in shared memory and scores nodes by table lookups.
 // A team's share of scoring the n nodes in slot[0..n): blocks of slot_block nodes in turn, each
 // staged and scored by one warp, totals into dist[0..n).  Block b takes the rows from b * SB mod STAGE_ROWS
 // of the staging area; the team's size divides their number, so the rows of a warp are its own.
@@ -1157,6 +1157,8 @@ __device__ __forceinline__ void score_team(const CT *C1s, uint8_t *stage, const 
 // others stage and score their share of each step's nodes (between two named barriers).  It
 // shortens a step, which bounds a small batch (16 queries 247 -> 227 us, one 94 -> 84), and wastes
 // issue slots in a large one.
+// TAB (the table form, LC_LUT_TABLE): no codebook; each warp keeps its query's ADC table
+// [256][M1] (FP16, built by table_kernel) in shared memory and scores nodes by table lookups.
 // BATCH: beam > 1.  The plain walk is an instantiation of its own: it visits one row and merges at
 // most 32 candidates a step, and the step's code has to stay small (the instruction cache bounds
 // it: with the code for four rows beside its own the plain walk of 10k queries took 908 and not
