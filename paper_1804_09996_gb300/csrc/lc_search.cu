@@ -839,7 +839,7 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     // block: 329 and 303 us at 1,459, 382 and 297 at 1,824 (20,000 x 96)
     const int64_t in_flight = (int64_t)P.grid * P.wpc;
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
-                (sp->order == LC_ORDER_ALWAYS || (sp->order == LC_ORDER_AUTO && nq >= in_flight + in_flight / 8));
+                (sp->order == LC_ORDER_ALWAYS || (sp->order == LC_ORDER_AUTO && nq >= in_flight + (in_flight + 7) / 8));
     P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
     if (P.ordered) {
         // the descent launch: its own kernel, many more warps (no level-0 state)
