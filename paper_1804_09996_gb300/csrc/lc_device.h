@@ -120,6 +120,7 @@ struct SearchPlan {
     int rw = 0, rgrid = 0, rteam = 1;    // refine: warps per CTA, CTAs, warps per query
     size_t rsm = 0;
     bool rboth = false;                  // both codebooks in shared memory
+    bool rearly = false;                 // refine: may start while the walk is there
     bool ordered = false;                // two walk launches, level 0 in decreasing entry distance
     bool tab = false;                    // table form: table_kernel, then the walk's table instantiation
     size_t tab_elems = 0;                // FP16 table entries of the batch

@@ -717,6 +717,16 @@ static RefineFn refine_kernel_for(bool both, int d, bool prod)
     return both ? (prod ? pick(T{}, T{}) : pick(T{}, F{})) : (prod ? pick(F{}, T{}) : pick(F{}, F{}));
 }
 
+// The shared memory that an SM sets aside for blocks of `smem` bytes, `ctas` at a time (KB; the rest of
+// its 256 KB is L1).
+static int smem_split(size_t smem, int64_t ctas)
+{
+    const size_t need = (smem + 1024) * (size_t)ctas;                // (1 KB per block is the system's)
+    for (int kb : {8, 16, 32, 64, 100, 132, 164, 196})
+        if (need <= (size_t)kb * 1024) return kb;
+    return 228;
+}
+
 lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params *sp, SearchPlan *pl,
                       bool allow_order)
 {
@@ -829,6 +839,13 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P.rw * 32, P.rsm);
         const int64_t teams = P.rw / P.rteam, need = (nq + teams - 1) / teams;
         P.rgrid = (int)std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * dv->num_sms);
+        // The re-rank may start while the walk is there (run_search), but an SM then keeps the walk's
+        // split of its memory.  Where C2 is read through L1, not if that leaves less L1 than the
+        // re-rank would have alone: 20,000 queries, d = 128, R = 10, with 28 KB and not 60 KB of L1: 702
+        // us and not 395; whole searches 1,848 -> 1,592 us, with beam 2 and R = 30 3,051 -> 2,254.  (Where
+        // it loses none, an early start saves 2 to 4 us of small batches.)
+        auto ctas = [&](int64_t grid) { return (grid + dv->num_sms - 1) / dv->num_sms; };
+        P.rearly = P.rboth || smem_split(P.smem, ctas(P.grid)) <= smem_split(P.rsm, ctas(P.rgrid));
     }
     // ordered search: worth its two extra launches once an eighth of the walks take a second query.
     // Query order against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500
@@ -918,12 +935,10 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     // large batches: the re-rank takes the queries as their walks end, on the SMs that have no more
     // (at 10k queries an SM is idle for a tenth of the walk launch while the longest walks end, and
     // the re-rank mostly fits into that: 721 -> 654 us for the batched FP16 search, 857 -> 781 us for
-    // the plain one, launch latencies included).  Not a re-rank that reads C2 through L1: started while
-    // the walk is there, an SM keeps the walk's split of its memory (228 KB shared, 28 KB of L1) where the
-    // re-rank alone gets 60 KB of L1, and takes 702 us in place of 395 (20,000 queries, d = 128, R = 10).
-    // It is launched when the walk has ended, by teams where those are faster (whole searches of 20,000
-    // queries at d = 128: 1,848 -> 1,592 us, with beam 2 and R = 30 3,051 -> 2,254)
-    const bool overlap = P.ordered && P.refine && P.rboth && !profile;
+    // the plain one, launch latencies included).  Not where it would lose L1 (P.rearly), nor where it reads
+    // C2 through L1 and is long enough for teams: d = 128, R = 100, 2,700 queries take 839 us so, 1,132 by
+    // one warp each beside the walk
+    const bool overlap = P.ordered && P.refine && P.rearly && (P.rboth || P.rteam == 1) && !profile;
     if (ce == cudaSuccess && P.tab) {
         // the batch's ADC tables on the tensor cores, from y'
         table_kernel<<<(unsigned)((nq + TAB_WARPS * 8 - 1) / (TAB_WARPS * 8)), TAB_WARPS * 32, 0, st>>>(
@@ -990,7 +1005,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
             ra.head = wa.done_tail + 1;
         }
         auto kern = refine_kernel_for(P.rboth, dv->d, dv->bM > 1);
-        ce = launch(kern, P.rgrid, P.rw * 32, P.rsm, st, P.rboth && !profile, ra);
+        ce = launch(kern, P.rgrid, P.rw * 32, P.rsm, st, P.rearly && !profile, ra);
         if (ce != cudaSuccess) {
             set_error("refine kernel launch failed: %s", cudaGetErrorString(ce));
             return LC_ERR_CUDA;
