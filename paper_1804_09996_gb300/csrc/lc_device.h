@@ -121,6 +121,7 @@ struct SearchPlan {
     size_t rsm = 0;
     bool rboth = false;                  // both codebooks in shared memory
     bool rearly = false;                 // refine: may start while the walk is there
+    bool overlap = false;                // refine: takes the queries as their walks end
     bool ordered = false;                // two walk launches, level 0 in decreasing entry distance
     bool tab = false;                    // table form: table_kernel, then the walk's table instantiation
     size_t tab_elems = 0;                // FP16 table entries of the batch

@@ -823,11 +823,12 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         // teams: the number of warps per query that ends first, counted in candidates per warp: rounds
         // of queries times the candidates of a team's busiest warp and its overhead (about two)
         const int groups = (P.R + REF_CH - 1) / REF_CH;
-        int64_t best = INT64_MAX;
+        int64_t best = 0;
         for (int t = 1; t <= std::min(P.rw, groups); t++) {
             const int64_t per_round = (int64_t)(P.rw / t) * dv->num_sms, rounds = (nq + per_round - 1) / per_round;
             const int64_t cost = rounds * (std::min(P.R, (groups + t - 1) / t * REF_CH) + 2);
-            if (cost < best) { best = cost; P.rteam = t; }
+            if (t == 1) best = cost - cost / 32;         // (a round more or less of large batches is no reason)
+            else if (cost < best) { best = cost; P.rteam = t; }
         }
         P.rsm = cb + per * P.rw;
         auto kern = refine_kernel_for(P.rboth, dv->d, dv->bM > 1);
@@ -839,13 +840,6 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P.rw * 32, P.rsm);
         const int64_t teams = P.rw / P.rteam, need = (nq + teams - 1) / teams;
         P.rgrid = (int)std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * dv->num_sms);
-        // The re-rank may start while the walk is there (run_search), but an SM then keeps the walk's
-        // split of its memory.  Where C2 is read through L1, not if that leaves less L1 than the
-        // re-rank would have alone: 20,000 queries, d = 128, R = 10, with 28 KB and not 60 KB of L1: 702
-        // us and not 395; whole searches 1,848 -> 1,592 us, with beam 2 and R = 30 3,051 -> 2,254.  (Where
-        // it loses none, an early start saves 2 to 4 us of small batches.)
-        auto ctas = [&](int64_t grid) { return (grid + dv->num_sms - 1) / dv->num_sms; };
-        P.rearly = P.rboth || smem_split(P.smem, ctas(P.grid)) <= smem_split(P.rsm, ctas(P.rgrid));
     }
     // ordered search: worth its two extra launches once an eighth of the walks take a second query.
     // Query order against ordered on 1M x 96, ef 64 (3,040 walks in flight): 531 and 527 us at 2,500
@@ -858,6 +852,30 @@ lc_status plan_search(const DeviceIndex *dv, int64_t nq, const lc_search_params 
     P.ordered = allow_order && nq <= INT32_MAX && dv->n > 0 &&
                 (sp->order == LC_ORDER_ALWAYS || (sp->order == LC_ORDER_AUTO && nq >= in_flight + (in_flight + 7) / 8));
     P.ord_elems = P.ordered ? (size_t)nq * 5 + 2 : 0;
+    // The re-rank may start while the walk is there, but an SM then keeps the walk's split of its memory.
+    // Where C2 is read through L1 that may leave less L1 than the re-rank would have alone (d = 128: 28 KB
+    // and not 60), which costs some 1.3 ns a candidate; without such a loss an early start is free and saves
+    // 2 to 4 us of small batches.  In an ordered search the re-rank may also take the queries as their walks
+    // end, on the SMs that have no more (at 10k queries an SM is idle for a tenth of the walk launch while the
+    // longest walks end, and the re-rank mostly fits into that: 721 -> 654 us for the batched FP16 search,
+    // 857 -> 781 us for the plain one, launch latencies included).  That time is worth a loss of L1 for few
+    // candidates; it is longer at a large efSearch, with one expansion a step and on the full decode.
+    // Plain against overlapped, 1M x 128, R = 10: efSearch 64, beam 4 893 and 957 us at 9,000 queries, 1,723
+    // and 1,916 at 20,000; beam 1 1,303 and 1,297, 2,535 and 2,673; efSearch 256, beam 4 2,596 and 2,511,
+    // 4,983 and 5,047; each query its own efSearch up to 256 1,593 and 1,466, 2,733 and 2,763; efSearch 32,
+    // full decode 556 and 507 at 3,000, 1,255 and 1,293 at 10,000.  In another process, its memory elsewhere, the
+    // plain re-rank of 20,000 queries took 475 us and not 399 (2,807 and 2,761), so the line is drawn where
+    // plain is no slower there either.  By teams (which one warp per query beside the walk would replace)
+    // it lies lower: R = 100, efSearch 64, 2,700 queries 839 and 1,132, but R = 32, efSearch up to 256 each,
+    // beam 1, 5,200 queries 2,028 and 1,930
+    if (P.refine) {
+        auto ctas = [&](int64_t grid) { return (grid + dv->num_sms - 1) / dv->num_sms; };
+        const int64_t few = P.rteam > 1 ? 1000 * (int64_t)(P.efp - 64)
+                                        : 1000 * (int64_t)P.efp + (P.beam == 1 ? 65000 : P.full ? 20000 : 0);
+        const bool beside = P.ordered && nq * P.R <= few;
+        P.rearly = P.rboth || beside || smem_split(P.smem, ctas(P.grid)) <= smem_split(P.rsm, ctas(P.rgrid));
+        P.overlap = P.ordered && P.rearly && (P.rboth || P.rteam == 1 || beside);
+    }
     if (P.ordered) {
         // the descent launch: its own kernel, many more warps (no level-0 state)
         WalkArgs wd{};
@@ -932,13 +950,7 @@ lc_status run_search(DeviceIndex *dv, const SearchPlan &P, const float *dq, int6
     // each kernel may start before the one ahead of it has ended, where that is a kernel which lets
     // it (not with the events of a profiled search between them)
     const bool pdl = !rotated && !P.tab && !profile;
-    // large batches: the re-rank takes the queries as their walks end, on the SMs that have no more
-    // (at 10k queries an SM is idle for a tenth of the walk launch while the longest walks end, and
-    // the re-rank mostly fits into that: 721 -> 654 us for the batched FP16 search, 857 -> 781 us for
-    // the plain one, launch latencies included).  Not where it would lose L1 (P.rearly), nor where it reads
-    // C2 through L1 and is long enough for teams: d = 128, R = 100, 2,700 queries take 839 us so, 1,132 by
-    // one warp each beside the walk
-    const bool overlap = P.ordered && P.refine && P.rearly && (P.rboth || P.rteam == 1) && !profile;
+    const bool overlap = P.overlap && !profile;          // the re-rank takes the queries as their walks end
     if (ce == cudaSuccess && P.tab) {
         // the batch's ADC tables on the tensor cores, from y'
         table_kernel<<<(unsigned)((nq + TAB_WARPS * 8 - 1) / (TAB_WARPS * 8)), TAB_WARPS * 32, 0, st>>>(

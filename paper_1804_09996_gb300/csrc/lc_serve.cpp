@@ -181,6 +181,7 @@ lc_status plan_batch(lc_server *s, Batch &b)
         // for the re-rank waits until it is idle first (300 requests of 300 queries, 16 outstanding,
         // d = 128: 18.3 ms, 20.2 with the late start of plan_search)
         b.plan.rearly = true;
+        b.plan.overlap |= b.plan.ordered && b.plan.refine && (b.plan.rboth || b.plan.rteam == 1);
         if (b.need <= s->budget || b.reqs.size() > 1) return LC_OK;
         if (b.plan.wpc > 1) b.sp.warps = b.plan.wpc > 16 ? 16 : b.plan.wpc / 2;
         else if (b.plan.ordered) b.sp.order = LC_ORDER_NEVER;
