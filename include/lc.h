@@ -111,9 +111,10 @@ typedef struct {
     int visited_log; /* 0: automatic; 10..14: the per-query visited table in shared memory has
                         2^visited_log entries (ids beyond three quarters of it go to a table
                         in global memory, see spill_log).  Automatic limits are held in tags of
-                        16 bits up to 2^25 vectors; where visited_log or spill_log is set, and
-                        above, the table holds 32-bit ids: the same set and results in nearly
-                        twice the shared memory, so fewer queries in flight */
+                        16 bits up to 2^25 vectors (2^24 where max(efSearch, k) is at most
+                        32); where visited_log or spill_log is set, and above, the table holds
+                        32-bit ids: the same set and results in nearly twice the shared memory,
+                        so fewer queries in flight */
     int beam;        /* LC_MODE_BATCHED: expansions per step, 2..8 (ignored in PLAIN mode) */
     int max_dist;    /* search-time cap T (Section 3.1): 0 = none; > 0: the level-0 search stops
                         before an expansion once T distances have been computed there */
